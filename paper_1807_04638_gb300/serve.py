@@ -153,7 +153,8 @@ class Server:
         self.max_inflight = int(max_inflight)
         self.device = torch.device("cuda", device)
         self.lock = threading.Condition()
-        self.inflight = 0
+        self.inflight = 0   # slots taken (a finished request's until it is retired)
+        self.done: List[tuple] = []  # finished, not yet retired: (request, handle, sticky status)
         self.results: Dict[int, Result] = {}
         self.t0 = None
         self.threads: List[threading.Thread] = []
@@ -197,7 +198,7 @@ class Server:
                 res.finished = time.perf_counter() - self.t0
                 with self.lock:
                     self.pool.cancel(hb)
-                    self.inflight -= 1
+                    self.done.append((req, None, 0))
                     self.lock.notify_all()
                 return
         h, _ = hb
@@ -221,12 +222,22 @@ class Server:
             if sticky != 0:  # a failed handle is not reused; closed outside the lock
                 h.close()
             with self.lock:
+                self.done.append((req, hb, sticky))
+                self.lock.notify_all()
+
+    def _retire(self):
+        """Called with the lock held: finished requests give up their slots,
+        and their handles go to the pool (or leave it, if they failed).  The
+        admission loop does this at the next admission, when a slot or a
+        handle is wanted; a finished worker only says so."""
+        for req, hb, sticky in self.done:
+            if hb is not None:
                 if sticky != 0:
                     self.pool.drop(hb)
                 else:
                     self._release_handle(req, hb)
-                self.inflight -= 1
-                self.lock.notify_all()
+            self.inflight -= 1
+        self.done.clear()
 
     def _admit_loop(self, pending: List[Request]):
         """Admit requests in arrival order as slots and memory free up."""
@@ -239,21 +250,31 @@ class Server:
                 i += 1
             admitted_any = False
             with self.lock:
-                while backlog and self.inflight < self.max_inflight:
+                while backlog:
+                    if self.inflight >= self.max_inflight:
+                        self._retire()
+                        if self.inflight >= self.max_inflight:
+                            break
                     req = backlog[0]
                     if req.deadline_s is not None and now - req.arrival > req.deadline_s:
                         backlog.pop(0)
                         r = self.results[req.rid]
                         r.status, r.finished = "error: admission deadline exceeded", now
                         continue
+                    # the request takes its slot, then the finished ones give up theirs
+                    self.inflight += 1
+                    self.peak_inflight = max(self.peak_inflight, self.inflight)
+                    self._retire()
                     try:
                         hb = self._reserve_handle(req)
                     except Exception as e:
+                        self.inflight -= 1
                         backlog.pop(0)
                         r = self.results[req.rid]
                         r.status, r.finished = f"error: {e}", now
                         continue
                     if hb is None:
+                        self.inflight -= 1
                         if self.inflight == 0:   # can never fit
                             backlog.pop(0)
                             r = self.results[req.rid]
@@ -261,8 +282,6 @@ class Server:
                             continue
                         break
                     backlog.pop(0)
-                    self.inflight += 1
-                    self.peak_inflight = max(self.peak_inflight, self.inflight)
                     self.results[req.rid].admitted = now
                     t = threading.Thread(target=self._run, args=(req, hb), daemon=True)
                     self.threads.append(t)
@@ -281,6 +300,8 @@ class Server:
         self._admit_loop(reqs)
         for t in self.threads:
             t.join()
+        with self.lock:
+            self._retire()
         return [self.results[r.rid] for r in requests]
 
     def close(self):
