@@ -148,20 +148,19 @@ def workload_inputs(n=N128, seed=1):
 
 
 # DRAM traffic per launch of the stage kernels, from an ncu capture
-# (profiles/fused_stages_128cubed_f32_ncu.md; one launch is one stage over the
+# (profiles/band_form_128cubed_f32_ncu.md; one launch is one stage over the
 # whole grid, the same at every nt), valid only for the kernel sources it was
 # measured on: reported as null once the sources change.
-TRAFFIC = {"digest": "d02ac607bd11f0f5", "adjoint_stage_fused": 359.7e6, "tangent_stage_fused": 386.5e6}
+TRAFFIC = {"digest": "d18a50554c362bf5", "adjoint_stage_fused": 186.4e6, "tangent_stage_fused": 197.0e6}
 
 
 def kernel_digest():
-    """Digest of the pass and stage-kernel sources (the dominant kernel
-    classes and their job layout): a stored DRAM-traffic figure holds only
-    for this digest."""
+    """Digest of the stage-kernel sources (the dominant kernel classes): a
+    stored DRAM-traffic figure holds only for this digest."""
     import hashlib
     h = hashlib.sha1()
     csrc = os.path.join(ROOT, "paper_1807_04638_gb300", "csrc")
-    for f in ("common.cuh", "fft_fast.cuh", "fft_kernels.cuh", "fused_stage.cuh"):
+    for f in ("common.cuh", "radix.cuh", "stage.cuh"):
         with open(os.path.join(csrc, f), "rb") as fh:
             h.update(fh.read())
     return h.hexdigest()[:16]

@@ -19,7 +19,16 @@ OUT_DIR = os.path.join(HERE, "lib")
 BUILD_DIR = os.path.join(HERE, "_build")
 LIB = os.path.join(OUT_DIR, "liblddmm.so")
 
-SOURCES = ["capi.cu", "engine_f64.cu", "engine_f32.cu", "noalloc.cu", "probe.cu"]
+# (source, object, defines): the passes are compiled once per number type, the
+# stage kernels once per number type and last radix, the kernels of a compiled
+# length once per length
+SOURCES = [(f"{s}.cu", f"{s}_{t}.o", (f"-DLDDMM_T={t}",))
+           for s in ("gen_pass", "fast_pass", "plane") for t in ("double", "float")]
+SOURCES += [(f"{s}.cu", f"{s}.o", ()) for s in ("engine_f32", "engine_f64", "noalloc", "capi", "probe")]
+SOURCES += [("stage_radix.cu", f"stage_{t}_{p}.o", (f"-DLDDMM_STAGE_T={t}", f"-DLDDMM_STAGE_P={p}"))
+            for t, ps in (("float", (6, 5, 4, 3)), ("double", (10, 9, 8, 6, 5, 4))) for p in ps]
+STAGE_LENGTHS = [384, 320, 300, 288, 270, 256, 250, 243, 240, 225, 216, 200, 192, 180, 162, 160, 150, 144, 135, 128, 125, 120, 108, 100, 96, 90, 81, 80, 75, 72, 64, 60, 54, 50, 48, 45, 40, 36, 32, 30, 27, 25, 24, 20, 18, 16]
+SOURCES += [("stage_length.cu", f"stage_n{n}.o", (f"-DLDDMM_STAGE_N={n}",)) for n in STAGE_LENGTHS]
 ARCH = ["-gencode", "arch=compute_103a,code=sm_103a"]
 
 
@@ -42,13 +51,13 @@ def build(verbose: bool = False, extra_flags=()) -> str:
     os.makedirs(BUILD_DIR, exist_ok=True)
     procs = []
     objs = []
-    for src in SOURCES:
-        obj = os.path.join(BUILD_DIR, src.replace(".cu", ".o"))
+    for src, name, defines in SOURCES:
+        obj = os.path.join(BUILD_DIR, name)
         objs.append(obj)
-        cmd = [nvcc, *_flags(extra_flags), "-c", os.path.join(CSRC, src), "-o", obj]
+        cmd = [nvcc, *_flags(extra_flags), *defines, "-c", os.path.join(CSRC, src), "-o", obj]
         if verbose:
             print(" ".join(cmd), flush=True)
-        procs.append((src, subprocess.Popen(cmd, stdout=subprocess.PIPE, stderr=subprocess.STDOUT)))
+        procs.append((name, subprocess.Popen(cmd, stdout=subprocess.PIPE, stderr=subprocess.STDOUT)))
     failed = []
     for src, p in procs:
         out, _ = p.communicate()

@@ -33,11 +33,15 @@
 #include <nvtx3/nvToolsExt.h>
 
 #include "common.cuh"
-#include "fft_fast.cuh"
+#include "fast_pass.cuh"
 #include "fft_kernels.cuh"
 #include "fused_stage.cuh"
+#include "gen_launch.cuh"
+#include "launch_util.cuh"
 #include "lddmm.h"
+#include "plane.cuh"
 #include "pw_kernels.cuh"
+#include "stage_dispatch.cuh"
 
 namespace lddmm {
 
@@ -53,11 +57,13 @@ struct NvtxRange {
 
 // Kernel classes for the optional CUDA-event profiler.
 enum KClass { KC_AX0 = 0, KC_AX1, KC_AX2, KC_ADSTAR, KC_TANPW, KC_ADJPW, KC_SL, KC_WARP, KC_RED, KC_SPEC, KC_MISC,
-              KC_SCAN, KC_TANF, KC_ADJF, KC_COUNT };
+              KC_SCAN, KC_TANF, KC_ADJF, KC_SHF, KC_PLI, KC_PLF, KC_STEP, KC_TAN64,
+              KC_ADJ64, KC_COUNT };
 static const char* const kclass_names[KC_COUNT] = {
     "fft_axis0_c2c", "fft_axis1_c2c", "fft_axis2_r2c_c2r", "adstar_pointwise", "tangent_pointwise",
     "adjoint_pointwise", "sl_map_step", "warp", "reduction", "spectral_combine", "misc_pointwise",
-    "input_scan", "tangent_stage_fused", "adjoint_stage_fused"};
+    "input_scan", "tangent_stage_fused", "adjoint_stage_fused", "shoot_stage_fused", "fft_plane_inverse",
+    "fft_plane_forward", "spectral_step", "tangent_stage_fp64", "adjoint_stage_fp64"};
 
 struct EngineBase {
     virtual ~EngineBase() {}
@@ -159,13 +165,13 @@ inline Layout layout_for(const Dims& d, const lddmm_params* p, size_t tsize) {
     Layout L;
     // pool + vhat(6) + v0hat(3) + v0full(3) + R1(3) + tan(12) + tb(6) + adj(12) + adja(6) + dhat(3) + tmp(3)
     L.spec_fields = POOL + 6 + 3 + 3 + 3 + 12 + 6 + 12 + 6 + 3 + 3;
-    // vfin(6) + u(6) + scratch + m1(1) + gm1(3) + r(1) + Lv0(3) + PCG (x r z p q g vt: 21)
+    // vfin(6) + u(6) + scratch + m1(1) + gm1(3) + PCG (x r z p q g vt: 21)
     // + FP32 copies of the last two stage-1 velocities for the map transport (6)
     const bool bf16 = p->state_dtype == LDDMM_BF16;
     const int cpe = p->checkpoint_every <= 1 ? p->nt : std::min(p->checkpoint_every, p->nt);
     const bool ckpt = cpe < p->nt;
     const int nseg = (p->nt + cpe - 1) / cpe;
-    L.real_fields = 6 + 6 + RSCR + 1 + 3 + 1 + 3 + 21 + 6;
+    L.real_fields = 6 + 6 + RSCR + 1 + 3 + 21 + 6;
     // exact discrete gradient: every map u_k, every dE/dv_k, two dE/du buffers
     if (p->gradient_mode == LDDMM_GRAD_DISCRETE) L.real_fields += (size_t)6 * (p->nt + 1) + 6;
     if (ckpt) L.spec_fields += (size_t)3 * nseg;  // spectral v at the checkpoints
@@ -205,8 +211,9 @@ inline bool force_no_graph() {
     const char* e = getenv("LDDMM_NO_GRAPH");
     return e && e[0] == '1';
 }
-// LDDMM_FULL_BAND=1 transforms every spectral line even where the 2/3-rule
-// band makes most of them zero; used to cross-check the band-limited passes.
+// LDDMM_FULL_BAND=1 runs the Jacobi sweeps through the separate passes and
+// transforms every spectral line even where the 2/3-rule band makes most of
+// them zero; used to cross-check the band-limited passes.
 inline bool force_full_band() {
     const char* e = getenv("LDDMM_FULL_BAND");
     return e && e[0] == '1';
@@ -234,143 +241,8 @@ inline std::vector<int> radix_plan(int n) {
     return r;
 }
 
-// The dynamic shared-memory limit of a kernel is process-wide: every site that
-// raises it sets the device's opt-in maximum, so that a handle (or call) for a
-// smaller grid never lowers the limit under a concurrent launch of a larger one.
-inline int smem_optin_max() {
-    int dev = 0, v = 48 * 1024;
-    if (cudaGetDevice(&dev) == cudaSuccess) cudaDeviceGetAttribute(&v, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev);
-    return v;
-}
-template <class K>
-inline bool raise_smem_limit(K kernel, size_t need) {
-    const int mx = smem_optin_max();
-    if ((size_t)mx < need) return false;
-    if (cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, mx) == cudaSuccess) return true;
-    cudaGetLastError();  // a refusal must not stay pending: the caller falls back to another kernel
-    return false;
-}
-
-// Ask for the smallest shared-memory carveout that holds `blocks` resident
-// blocks of `bytes` dynamic shared memory each, so that the rest of the SM's
-// unified L1/shared storage stays L1 (a hint: the driver rounds it up to a
-// split it supports).
-template <class K>
-inline void prefer_l1(K kernel, size_t bytes, int blocks) {
-    int dev = 0, per_sm = 0, resv = 0;
-    if (cudaGetDevice(&dev) != cudaSuccess ||
-        cudaDeviceGetAttribute(&per_sm, cudaDevAttrMaxSharedMemoryPerMultiprocessor, dev) != cudaSuccess ||
-        cudaDeviceGetAttribute(&resv, cudaDevAttrReservedSharedMemoryPerBlock, dev) != cudaSuccess || per_sm <= 0) {
-        cudaGetLastError();
-        return;
-    }
-    const size_t need = (size_t)blocks * (bytes + (size_t)resv);
-    const int pct = (int)std::min<size_t>(100, (need * 100 + (size_t)per_sm - 1) / (size_t)per_sm);
-    if (cudaFuncSetAttribute(kernel, cudaFuncAttributePreferredSharedMemoryCarveout, pct) != cudaSuccess)
-        cudaGetLastError();  // a hint only
-}
-
-// Grid of a persistent pass: `per_sm` resident blocks per SM, never more
-// blocks than work items.
-inline int persistent_grid(int items, int per_sm = 3) {
-    static int sms = 0;
-    if (!sms) {
-        int dev = 0;
-        cudaGetDevice(&dev);
-        cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-        if (sms <= 0) sms = 152;
-    }
-    return std::max(1, std::min(items, per_sm * sms));
-}
-
-// Launch of the register-blocked passes for the compiled line lengths.
-template <class T> struct FastPass {
-    // the persistent axis-2 kernel's shared-memory limit is raised (per N)
-    template <int N> static bool& a2p_ready() {
-        static bool v = false;
-        return v;
-    }
-    // The persistent axis-2 kernel takes full tiles of r2 rows, one input per
-    // inverse job, and 16-byte aligned inputs (its copies are 16-byte
-    // cp.async of whole rows or plane segments).
-    static bool axis2p_fits(const PassParams<T>& pp, int nj, size_t rows, int r2) {
-        if (rows % (size_t)r2 != 0 || (rows / r2) * (size_t)nj >= (1u << 24)) return false;
-        for (int j = 0; j < nj; ++j) {
-            const PassJobT<T>& jb = pp.jobs[j];
-            if (pp.sign > 0 && jb.nin != 1) return false;
-            for (int i = 0; i < jb.nin; ++i)
-                if ((uintptr_t)jb.in[i] % 16 != 0) return false;
-        }
-        return true;
-    }
-    template <int N>
-    static bool go(int axis, int sign, PassParams<T>& pp, int nj, size_t rows, int n0, int n1, int n2h,
-                   cudaStream_t st, bool set_attr) {
-        (void)sign;
-        constexpr int TL = FAST_THREADS / (N / FastPlan<N>::E);
-        if (axis == 2) {
-            const size_t sm = fast_axis2_smem<T, N>();
-            constexpr bool PERS = sizeof(T) == 4 && FastPlan<N>::E <= 12;
-            if (set_attr) {
-                if constexpr (PERS) a2p_ready<N>() = raise_smem_limit(k_fast_axis2p<T, N>, fast_axis2p_smem<T, N>());
-                return raise_smem_limit(k_fast_axis2<T, N>, sm);
-            }
-            if constexpr (PERS) {
-                if (a2p_ready<N>() && axis2p_fits(pp, nj, rows, 2 * TL)) {
-                    const int ntiles = (int)(rows / (2 * TL));
-                    pp.fd_tiles = FastDiv((unsigned)ntiles);
-                    k_fast_axis2p<T, N><<<persistent_grid(ntiles * nj, A2P_BLOCKS), FAST_THREADS, fast_axis2p_smem<T, N>(),
-                                          st>>>(pp, ntiles);
-                    return true;
-                }
-            }
-            const int gx = (int)((rows + 2 * TL - 1) / (2 * TL));
-            k_fast_axis2<T, N><<<dim3(gx, nj), FAST_THREADS, sm, st>>>(pp);
-        } else if (axis == 1) {
-            const size_t sm = fast_c2c_smem<T, N>(1);
-            if (set_attr) {
-                if (!raise_smem_limit(k_fast_c2c<T, N, 1>, sm)) return false;
-                prefer_l1(k_fast_c2c<T, N, 1>, sm, FastOccC2C<T, N>::value);
-                return true;
-            }
-            (void)n2h;
-            const int ntiles = (int)(((size_t)pp.nb2 * n0 + TL - 1) / TL);
-            pp.fd_tiles = FastDiv((unsigned)ntiles);
-            pp.fd_n0 = FastDiv((unsigned)n0);
-            k_fast_c2c<T, N, 1><<<persistent_grid(ntiles * nj), FAST_THREADS, sm, st>>>(pp, ntiles);
-        } else {
-            const size_t sm = fast_c2c_smem<T, N>(0);
-            if (set_attr) {
-                if (!raise_smem_limit(k_fast_c2c<T, N, 0>, sm)) return false;
-                prefer_l1(k_fast_c2c<T, N, 0>, sm, FastOccC2C<T, N>::value);
-                return true;
-            }
-            const int tpk = (pp.c1 + TL - 1) / TL + (n1 - pp.s1 + TL - 1) / TL;
-            const int ntiles = pp.nb2 * tpk;
-            pp.fd_tiles = FastDiv((unsigned)ntiles);
-            pp.fd_tpk = FastDiv((unsigned)tpk);
-            k_fast_c2c<T, N, 0><<<persistent_grid(ntiles * nj), FAST_THREADS, sm, st>>>(pp, ntiles);
-        }
-        return true;
-    }
-    // n: the line length of this axis.  Returns false when no plan exists.
-    static bool launch(int n, int axis, int sign, PassParams<T>& pp, int nj, size_t rows, int n0, int n1, int n2h,
-                       cudaStream_t st, bool set_attr = false) {
-        switch (n) {
-            case 32: return go<32>(axis, sign, pp, nj, rows, n0, n1, n2h, st, set_attr);
-            case 64: return go<64>(axis, sign, pp, nj, rows, n0, n1, n2h, st, set_attr);
-            case 128: return go<128>(axis, sign, pp, nj, rows, n0, n1, n2h, st, set_attr);
-            case 256: return go<256>(axis, sign, pp, nj, rows, n0, n1, n2h, st, set_attr);
-            case 96: return go<96>(axis, sign, pp, nj, rows, n0, n1, n2h, st, set_attr);
-            case 160: return go<160>(axis, sign, pp, nj, rows, n0, n1, n2h, st, set_attr);
-            case 192: return go<192>(axis, sign, pp, nj, rows, n0, n1, n2h, st, set_attr);
-            default: return false;
-        }
-    }
-    static bool has(int n) { return n == 32 || n == 64 || n == 96 || n == 128 || n == 160 || n == 192 || n == 256; }
-};
-
-// Launch of the fused Jacobi stage kernels (FP32, n2 with an E = 8 plan).
+// Launch of the fused Jacobi stage kernels of the bfloat16-state form (n2 with
+// an E = 8 plan; the other forms run the stages of stage.cuh).
 struct FusedPass {
     static bool has(int n) { return n == 32 || n == 64 || n == 128 || n == 256; }
     static int tile_rows(int n) { return FAST_THREADS / (n / 8); }
@@ -397,8 +269,7 @@ struct FusedPass {
         }
     }
     static bool prepare(int n) {
-        return launch<float, 0>(n, FusedArgs{}, 0, true) && launch<float, 1>(n, FusedArgs{}, 0, true) &&
-               launch<__nv_bfloat16, 0>(n, FusedArgs{}, 0, true) && launch<__nv_bfloat16, 1>(n, FusedArgs{}, 0, true);
+        return launch<__nv_bfloat16, 0>(n, FusedArgs{}, 0, true) && launch<__nv_bfloat16, 1>(n, FusedArgs{}, 0, true);
     }
 };
 
@@ -448,7 +319,7 @@ class Engine : public EngineBase {
     int cpe = 1, nseg = 1, seg_res = -1;
     bool ckpt = false;
     C* cps = nullptr;
-    T *vfin, *ubuf[2], *rs, *m1, *gm1, *rbuf, *lv0, *vss[2] = {nullptr, nullptr};
+    T *vfin, *ubuf[2], *rs, *m1, *gm1, *vss[2] = {nullptr, nullptr};
     // exact discrete gradient: maps u_k (k = 0..nt), dE/dv_k, dE/du ping-pong
     T *ustore = nullptr, *vbar = nullptr, *ubar[2] = {nullptr, nullptr};
     bool exact_grad = false;
@@ -460,11 +331,22 @@ class Engine : public EngineBase {
     SpecTabs<T> tabs;
     int TLc[2], Pc[2], TL2, P2, Ph2;
     bool fast[3] = {false, false, false};
+    bool gen[2] = {false, false};  // C2C axes without a register-blocked plan: k_gen_c2c
+    RPlan gpl[2];
     // band-limited transforms (all three passes register-blocked, dealiasing on)
     bool band_ok = false;
     bool sl_staged = false;  // FP32 map steps use k_sl_step_staged
     bool fused = false;      // FP32 Jacobi stages use k_fused_stage
     int bnb2 = 0, bc1 = 0, bs1 = 0;
+    // band form (plane.cuh, stage.cuh): dealiasing on, states in the compute type
+    bool band_form = false;    // the shooting runs it
+    bool band_sweeps = false;  // the Jacobi sweeps too
+    Band bd;
+    RPlan rpl[3], rpl_st;
+    int st_lrb = 0, st_threads = 0, pl_tile[2] = {0, 0}, pl_threads = 0;
+    bool pl_split = false, pl_lines = false;
+    size_t st_smem = 0, pl_smem[4] = {0, 0, 0, 0};
+    T *Lt = nullptr, *Kt = nullptr;
     size_t smem_c[2], smem2;
     int pool_top = 0;
     bool lin_valid = false;
@@ -624,8 +506,6 @@ class Engine : public EngineBase {
         rs = carve<T>((size_t)RSCR * d.N);
         m1 = carve<T>(d.N);
         gm1 = carve<T>(3 * d.N);
-        rbuf = carve<T>(d.N);
-        lv0 = carve<T>(3 * d.N);
         px = carve<T>(3 * d.N);
         pr = carve<T>(3 * d.N);
         pz = carve<T>(3 * d.N);
@@ -708,6 +588,10 @@ class Engine : public EngineBase {
             fast[a] = FastPass<T>::has(ns[a]) && aligned && !force_generic_fft() &&
                       FastPass<T>::launch(ns[a], a, 0, dummy, 0, 0, 0, 0, 0, st, true);
         }
+        for (int a = 0; a < 2; ++a) {
+            gpl[a] = radix_plan3(ns[a]);
+            if (!fast[a] && gpl[a].n && !force_generic_fft()) gen[a] = GenPass<T>::prepare(a, gpl[a]);
+        }
         // the 2/3-rule band: k2 <= kcut2; k1 columns rounded outwards to even
         // indices (16-byte copies of FP32 pairs)
         bnb2 = std::min(tabs.kcut[2] + 1, d.n2h);
@@ -717,11 +601,13 @@ class Engine : public EngineBase {
         if constexpr (sizeof(T) == 4)
             sl_staged = !force_sl_gather() && raise_smem_limit(k_sl_step_staged<true>, SLBox<true>::SMEM) &&
                         raise_smem_limit(k_sl_step_staged<false>, SLBox<false>::SMEM);
-        band_ok = prm.dealias && fast[0] && fast[1] && fast[2] && !force_full_band() &&
-                  (bnb2 < d.n2h || bc1 < bs1);
+        band_ok = prm.dealias && (fast[0] || gen[0]) && (fast[1] || gen[1]) && !force_generic_fft() &&
+                  !force_full_band() && (bnb2 < d.n2h || bc1 < bs1);
         if constexpr (sizeof(T) == 4)
-            fused = band_ok && !force_unfused() && FusedPass::has(d.n2) && bnb2 == FusedPass::band_planes(d.n2) &&
+            fused = bf16 && band_ok && !force_unfused() && FusedPass::has(d.n2) && bnb2 == FusedPass::band_planes(d.n2) &&
                     d.rows % (size_t)FusedPass::tile_rows(d.n2) == 0 && FusedPass::prepare(d.n2);
+        band_form = prm.dealias && !bf16 && band_init();
+        band_sweeps = band_form && !force_unfused() && !force_full_band();
         LD_CK(cudaStreamSynchronize(st));
         return LDDMM_OK;
     }
@@ -776,6 +662,9 @@ class Engine : public EngineBase {
                 const int n = axis == 0 ? d.n0 : (axis == 1 ? d.n1 : d.n2);
                 PScope ps_(this, axis == 0 ? KC_AX0 : (axis == 1 ? KC_AX1 : KC_AX2), pass_bytes(axis, sign, pp_));
                 FastPass<T>::launch(n, axis, sign, pp_, nj, d.rows, d.n0, d.n1, d.n2h, st);
+            } else if (axis < 2 && gen[axis]) {
+                PScope ps_(this, axis == 0 ? KC_AX0 : KC_AX1, pass_bytes(axis, sign, pp_));
+                GenPass<T>::launch(axis, sign, pp_, nj, gpl[axis], st);
             } else if (axis == 2) {
                 pp_.TL = TL2;
                 pp_.P = P2;
@@ -835,19 +724,13 @@ class Engine : public EngineBase {
         }
     }
     // slot = <L v0, v0> (regulariser of the energy), from F(v0) in v0full
-    void reg_async(const T* v0, int slot) {
-        std::vector<SpecLin> srcs;
-        std::vector<InvReq> reqs;
-        for (int c = 0; c < 3; ++c) {
-            SpecLin s;
-            s.n = 1;
-            s.p[0] = v0full + c * d.NS;
-            s.c[0] = 1.0;
-            srcs.push_back(s);
-            reqs.push_back({c, sym(1.0, 1, -1), lv0 + c * d.N});
+    void reg_async(int slot) {
+        {
+            PScope ps_(this, KC_RED, 3.0 * d.NS * sizeof(C));
+            k_spec_energy<T><<<RED_BLOCKS, spec_comb_threads(d.n1), 0, st>>>(v0full, d.NS, tabs, d.n0, d.n1, d.n2h, partial);
         }
-        inverse(srcs, reqs);
-        dot_async(lv0, v0, 3 * d.N, slot, d.cell);
+        PScope ps_(this, KC_RED, 0.0);
+        k_finish<<<1, RED_THREADS, 0, st>>>(partial, RED_BLOCKS, 1, 0, 0, d.cell / (double)d.N, dres + slot);
     }
 
     // The axis-2 inputs of an inverse transform: request r reads spectrum
@@ -1153,10 +1036,13 @@ class Engine : public EngineBase {
     }
 
     // ------------------------------------------------------------ reductions
-    void dot_async(const T* a, const T* b, size_t n, int slot, double scale) {
+    // slot = scale * sum of a b (b null: a^2; diff: (a - b)^2)
+    void dot_async(const T* a, const T* b, size_t n, int slot, double scale, bool diff = false) {
         {
             PScope ps_(this, KC_RED, (double)(b ? 2 : 1) * n * sizeof(T));
-            k_dot_partial<T><<<RED_BLOCKS, RED_THREADS, 0, st>>>(a, b, n, partial);
+            if (!b) k_dot_partial<T, DOT_AA><<<RED_BLOCKS, RED_THREADS, 0, st>>>(a, b, n, partial);
+            else if (diff) k_dot_partial<T, DOT_DIFF><<<RED_BLOCKS, RED_THREADS, 0, st>>>(a, b, n, partial);
+            else k_dot_partial<T, DOT_AB><<<RED_BLOCKS, RED_THREADS, 0, st>>>(a, b, n, partial);
         }
         {
             PScope ps_(this, KC_RED, 0.0);
@@ -1179,8 +1065,8 @@ class Engine : public EngineBase {
         LD_CK(cudaStreamSynchronize(st));
         return LDDMM_OK;
     }
-    double dot_now(const T* a, const T* b, size_t n) {
-        dot_async(a, b, n, 63, d.cell);
+    double dot_now(const T* a, const T* b, size_t n, bool diff = false) {
+        dot_async(a, b, n, 63, d.cell, diff);
         if (fetch(63, 1) != LDDMM_OK) return NAN;
         return hres[63];
     }
@@ -1310,6 +1196,11 @@ class Engine : public EngineBase {
         if (!ckpt || seg_res == j) return;
         seg_res = j;
         const int k0 = j * cpe, k1 = std::min(prm.nt, k0 + cpe);
+        if (band_form) {
+            band_vec_copy(vhat[0], cps + (size_t)j * 3 * d.NS);
+            for (int k = k0; k < k1; ++k) band_shoot_step(k, false, false);
+            return;
+        }
         for (int k = k0; k < k1; ++k) {
             const C* cur = k == k0 ? cps + (size_t)j * 3 * d.NS : vhat[k % 2];
             shoot_step(k, cur, vhat[(k + 1) % 2], false, false);
@@ -1325,9 +1216,17 @@ class Engine : public EngineBase {
         const T ih0 = (T)(1.0 / d.h[0]), ih1 = (T)(1.0 / d.h[1]), ih2 = (T)(1.0 / d.h[2]);
         const int cubic = prm.interp == LDDMM_INTERP_CUBIC;
         fwd_vec(v0, v0full);
-        mask_copy(v0full, v0hat);
         cudaMemsetAsync(ubuf_at(0), 0, 3 * d.N * sizeof(T), st);
-        for (int k = 0; k < nt; ++k) {
+        if (band_form) band_copy<true>(v0full, vhat[0]);
+        else mask_copy(v0full, v0hat);
+        for (int k = 0; k < nt && band_form; ++k) {
+            if (ckpt && k % cpe == 0) {
+                band_vec_copy(cps + (size_t)(k / cpe) * 3 * d.NS, vhat[0]);
+                seg_res = k / cpe;
+            }
+            band_shoot_step(k, true, kinetic);
+        }
+        for (int k = 0; k < nt && !band_form; ++k) {
             C* cur = k == 0 ? v0hat : vhat[k % 2];
             C* nxt = vhat[(k + 1) % 2];
             if (ckpt && k % cpe == 0) {
@@ -1338,7 +1237,12 @@ class Engine : public EngineBase {
             shoot_step(k, cur, nxt, true, kinetic);
         }
         // v_nt, m_nt in real space, last map step
-        {
+        if (band_form) {
+            std::vector<BandReq> rq;
+            for (int c = 0; c < 3; ++c) rq.push_back({vhat[0] + c * d.NS, 0, nullptr, 1.0});
+            for (int c = 0; c < 3; ++c) rq.push_back({vhat[0] + c * d.NS, 0, Lt, 1.0});
+            band_to_real(rq, vfin);
+        } else {
             std::vector<SpecLin> srcs;
             std::vector<InvReq> reqs;
             for (int c = 0; c < 3; ++c) {
@@ -1355,7 +1259,7 @@ class Engine : public EngineBase {
         if (kinetic) dot_async(vfin + 3 * d.N, vfin, 3 * d.N, nt, d.cell);
         {
             PScope ps_(this, KC_SL, 12.0 * d.N * sizeof(T));
-            sl_step(gi, vss[(nt - 1) % 2], vfin, ubuf_at(nt - 1), ubuf_at(nt), (T)dt_, ih0, ih1, ih2, cubic);
+            sl_step(gi, vnat(nt - 1), vfin, ubuf_at(nt - 1), ubuf_at(nt), (T)dt_, ih0, ih1, ih2, cubic);
         }
     }
     T* u1() const { return ubuf_at(prm.nt); }
@@ -1384,6 +1288,10 @@ class Engine : public EngineBase {
     // tangent: from tan_[0] = (eta0, xi0); result in tan_[nt % 2]
     void tangent_sweep() {
         NvtxRange nr_("lddmm tangent sweep");
+        if (band_sweeps) {
+            band_tangent_sweep();
+            return;
+        }
         const double dt_ = dt();
         T* E = rs;                  // 24 fields
         T* X = rs + 24 * d.N;       // 12 fields
@@ -1463,7 +1371,7 @@ class Engine : public EngineBase {
     // axis-1/0 passes of the forward transform
     void fused_launch(FusedArgs& a, int sidx, int kind) {
         if constexpr (sizeof(T) == 4) {
-            a.states = bf16 ? (const void*)state_bf(sidx) : (const void*)state(sidx);
+            a.states = (const void*)state_bf(sidx);
             a.dk2 = (const float*)tabs.dk[2];
             a.tw = (const cpx<float>*)ax[2].tw;
             a.rows = (int)d.rows;
@@ -1473,14 +1381,8 @@ class Engine : public EngineBase {
             const double band = (double)bnb2 * d.rows * sizeof(C);
             const double bytes = 33.0 * band + 24.0 * d.N * state_elem() + (a.eta_src ? 3.0 * d.N * sizeof(T) : 0.0);
             PScope ps_(this, kind == 0 ? KC_TANF : KC_ADJF, bytes);
-            bool ok;
-            if (bf16) {
-                if (kind == 0) ok = FusedPass::launch<__nv_bfloat16, 0>(d.n2, a, st);
-                else ok = FusedPass::launch<__nv_bfloat16, 1>(d.n2, a, st);
-            } else {
-                if (kind == 0) ok = FusedPass::launch<float, 0>(d.n2, a, st);
-                else ok = FusedPass::launch<float, 1>(d.n2, a, st);
-            }
+            const bool ok = kind == 0 ? FusedPass::launch<__nv_bfloat16, 0>(d.n2, a, st)
+                                      : FusedPass::launch<__nv_bfloat16, 1>(d.n2, a, st);
             if (!ok) fail(LDDMM_ERR_DEVICE_CHECK);
         }
     }
@@ -1552,6 +1454,10 @@ class Engine : public EngineBase {
     // added to ybar_eta after the transposed step k (exact discrete gradient)
     void adjoint_sweep(const T* eta_src = nullptr) {
         NvtxRange nr_("lddmm adjoint sweep");
+        if (band_sweeps) {
+            band_adjoint_sweep(eta_src);
+            return;
+        }
         const double dt_ = dt();
         T* Y = rs;              // 6 fields
         T* G = rs + 6 * d.N;    // 36 fields
@@ -1630,7 +1536,378 @@ class Engine : public EngineBase {
             cur_i = 1 - cur_i;
         }
     }
-    C* adj_result() const { return adj[prm.nt % 2]; }
+    C* adj_result() const { return adj[band_sweeps ? 0 : prm.nt % 2]; }
+
+    // ------------------------------------------------------------ band form
+    // Buffers of the pool: planes into a stage, planes out of it, their band
+    // spectra, the half-transformed band of split planes, planes at the
+    // natural-layout boundary.
+    static constexpr int B_IN = 0, B_OUT = 14, B_SPEC = 28, B_MID = 44, B_NAT = 58;
+    bool band_init() {
+        const int ns[3] = {d.n0, d.n1, d.n2};
+        for (int a = 0; a < 3; ++a) {
+            rpl[a] = radix_plan3(ns[a]);
+            if (!rpl[a].n) return false;
+        }
+        memset((void*)&bd, 0, sizeof(bd));
+        bd.n0 = d.n0;
+        bd.n1 = d.n1;
+        bd.n2 = d.n2;
+        bd.kc0 = tabs.kcut[0];
+        bd.kc1 = tabs.kcut[1];
+        bd.kc2 = tabs.kcut[2];
+        bd.p0 = bd.kc0 + 1;
+        bd.b0 = 2 * bd.kc0 + 1;
+        bd.p1 = bd.kc1 + 1;
+        bd.b1 = 2 * bd.kc1 + 1;
+        bd.nb2 = bd.kc2 + 1;
+        bd.fb0 = FastDiv((unsigned)bd.b0);
+        bd.fb1 = FastDiv((unsigned)bd.b1);
+        bd.fn1 = FastDiv((unsigned)d.n1);
+        bd.b0p = (bd.b0 + 1) & ~1;
+        bd.size = (size_t)bd.nb2 * bd.b1 * bd.b0p;
+        const size_t mx = (size_t)smem_optin_max();
+        // stage kernel: 8 row pairs (FP32), or 16 rows and fewer of long lines (FP64)
+        constexpr bool f32 = sizeof(T) == 4;
+        rpl_st = stage_plan(!f32, d.n2);
+        if (!rpl_st.n) return false;
+        const int W = d.n2 / rpl_st.c;
+        st_lrb = f32 ? (stage_rb(d.n2, rpl_st.c) == 8 ? 3 : 2) : 4;
+        while (!f32 && st_lrb > 1 && (W << st_lrb) > STAGE_THREADS) --st_lrb;
+        st_threads = ((W << st_lrb) + 31) / 32 * 32;
+        st_smem = stage_smem(!f32, d.n2, st_lrb);
+        if (st_threads > (f32 ? STAGE2_THREADS : STAGE_THREADS) || st_smem > mx) return false;
+        StageArgs<T> sa;
+        sa.pl = rpl_st;
+        sa.rows = (int)d.rows;
+        sa.n2 = d.n2;
+        sa.nb2 = bd.nb2;
+        for (int kind = 0; kind < 3; ++kind)
+            if (!stage_launch(kind, sa, 0, 0, mx, st, true)) return false;
+        // axis-0 and axis-1 transforms: FP32 with compiled lengths, else both axes
+        // in one launch where a plane fits
+        if constexpr (f32) {
+            PlaneArgs<float> dummy;
+            pl_lines = true;
+            for (int mode = 0; mode < 4 && pl_lines; ++mode)
+                pl_lines = line_launch(mode == 0 || mode == 3 ? d.n1 : d.n0, mode, dummy, dim3(), st, true);
+        }
+        pl_smem[3] = plane_smem<T>(3, bd, 0);
+        pl_split = f32 || pl_smem[3] > mx;
+        pl_threads = !pl_split && pl_smem[3] > 112 * 1024 ? 512 : 256;
+        pl_tile[0] = pl_tile[1] = 16;
+        pl_smem[1] = plane_smem<T>(1, bd, pl_tile[0]);
+        pl_smem[2] = plane_smem<T>(2, bd, pl_tile[1]);
+        PlaneArgs<T> pa;
+        for (int ph = pl_split ? 1 : 3; ph <= (pl_split ? 2 : 3) && !pl_lines; ++ph)
+            for (int inverse = 0; inverse < 2; ++inverse)
+                if (!plane_kernel<T>(inverse != 0, ph, pa, dim3(), 0, pl_smem[ph], st, true)) return false;
+        // R1 is free in this form: it keeps the tables of L and K over the band
+        Lt = (T*)R1;
+        Kt = (T*)(R1 + d.NS);
+        k_band_tables<T><<<(unsigned)((bd.size + 255) / 256), 256, 0, st>>>(bd, d.len[0], d.len[1], d.len[2], prm.alpha,
+                                                                          prm.s, Lt, Kt);
+        return cudaGetLastError() == cudaSuccess;
+    }
+
+    // a real field of an inverse: scale [tab] times a component of the spectra
+    // at `in` (kind 0), i kappa . X (1), or component c of i kappa x X (2 + c)
+    struct BandReq {
+        const C* in;
+        int kind;
+        const T* tab;
+        double scale;
+    };
+    void plane_launch(bool inverse, PlaneArgs<T>& a, int nf, double bytes) {
+        a.bd = bd;
+        a.pl0 = rpl[0];
+        a.pl1 = rpl[1];
+        a.tw0 = (const C*)ax[0].tw;
+        a.tw1 = (const C*)ax[1].tw;
+        for (int q = 0; q < 3; ++q) a.dk[q] = tabs.dk[q];
+        a.cs = d.NS;
+        a.mid = pool[B_MID];
+        a.mids = (size_t)(pool[1] - pool[0]);
+        auto shape = [&](int ph) {
+            a.tile = pl_tile[ph - 1];
+            a.ft = FastDiv((unsigned)a.tile);
+            return (unsigned)(bd.nb2 * (((ph == 1 ? bd.b0 : d.n1) + a.tile - 1) / a.tile));
+        };
+        const int cls = inverse ? KC_PLI : KC_PLF;
+        const double half = 0.5 * bytes + (double)nf * bd.nb2 * d.n1 * bd.b0 * sizeof(C);
+        if constexpr (sizeof(T) == 4)
+            if (pl_lines) {
+                for (int q = 0; q < 2; ++q) {
+                    PScope ps_(this, cls, half);
+                    const int mode = (inverse ? 0 : 2) + q;
+                    const bool ax1 = mode == 0 || mode == 3;
+                    const unsigned pairs = (unsigned)((ax1 ? bd.b0 : d.n1) + 1) / 2;
+                    line_launch(ax1 ? d.n1 : d.n0, mode, a, dim3((pairs + LINE_RB - 1) / LINE_RB, bd.nb2, nf), st);
+                }
+                return;
+            }
+        if (!pl_split) {
+            PScope ps_(this, cls, bytes);
+            const dim3 g((unsigned)bd.nb2, (unsigned)nf);
+            plane_kernel<T>(inverse, 3, a, g, pl_threads, pl_smem[3], st);
+            return;
+        }
+        for (int q = 0; q < 2; ++q) {
+            PScope ps_(this, cls, half);
+            const int ph = inverse ? 1 + q : 2 - q;
+            const dim3 g(shape(ph), (unsigned)nf);
+            plane_kernel<T>(inverse, ph, a, g, pl_threads, pl_smem[ph], st);
+        }
+    }
+    // axis-1 and axis-0 inverse transforms of the requests into pool[first..]
+    void plane_inverse(const std::vector<BandReq>& rq, int first) {
+        PlaneArgs<T> a;
+        const double invN = 1.0 / (double)d.N;
+        double bytes = 0;
+        for (size_t j = 0; j < rq.size(); ++j) {
+            a.jobs[j].in = rq[j].in;
+            a.jobs[j].out = pool[first + j];
+            a.jobs[j].tab = rq[j].tab;
+            a.jobs[j].scale = (T)(rq[j].scale * invN);
+            a.jobs[j].kind = rq[j].kind;
+            bytes += (double)bd.nb2 * d.rows * sizeof(C) +
+                     (double)bd.size * (sizeof(C) * (rq[j].kind == 0 ? 1 : (rq[j].kind == 1 ? 3 : 2)) + (rq[j].tab ? sizeof(T) : 0));
+        }
+        plane_launch(true, a, (int)rq.size(), bytes);
+    }
+    // axis-0 and axis-1 forward transforms of pool[first..] into out[0..nf)
+    void plane_forward(int first, int nf, C* const* out) {
+        PlaneArgs<T> a;
+        for (int j = 0; j < nf; ++j) {
+            memset((void*)&a.jobs[j], 0, sizeof(a.jobs[j]));
+            a.jobs[j].in = pool[first + j];
+            a.jobs[j].out = out[j];
+        }
+        plane_launch(false, a, nf, (double)nf * ((double)bd.nb2 * d.rows + bd.size) * sizeof(C));
+    }
+    // axis-2 inverse of planes pool[first..] into the natural layout
+    void nat_inverse(int first, int nf, T* out) {
+        std::vector<PassJob> jobs;
+        for (int j = 0; j < nf; ++j) {
+            PassJob q = blank();
+            q.nin = q.nout = 1;
+            q.in[0] = pool[first + j];
+            q.isym[0] = q.osym[0] = sym(1.0, 0, -1);
+            q.out[0] = out + (size_t)j * d.N;
+            jobs.push_back(q);
+        }
+        launch(2, +1, jobs, true);
+    }
+    void band_to_real(const std::vector<BandReq>& rq, T* out) {
+        plane_inverse(rq, B_IN);
+        nat_inverse(B_IN, (int)rq.size(), out);
+    }
+    // three real components -> band spectrum (both forms: only the band is used)
+    void band_fwd_vec(const T* in, C* out) {
+        if (!band_sweeps) {
+            fwd_vec(in, out, 1.0, 0, true);
+            return;
+        }
+        std::vector<PassJob> jobs;
+        C* o[3];
+        for (int c = 0; c < 3; ++c) {
+            PassJob q = blank();
+            q.nin = q.nout = 1;
+            q.in[0] = in + (size_t)c * d.N;
+            q.isym[0] = sym(1.0, 0, -1);
+            q.out[0] = pool[B_NAT + c];
+            o[c] = out + c * d.NS;
+            jobs.push_back(q);
+        }
+        launch(2, -1, jobs, true);
+        plane_forward(B_NAT, 3, o);
+    }
+    // full spectrum -> band (with P), or band -> full (zeros outside); 3 components
+    template <bool TOBAND> void band_copy(const C* src, C* dst) {
+        const size_t n = TOBAND ? bd.size : d.NS;
+        PScope ps_(this, KC_SPEC, 3.0 * (bd.size + n) * sizeof(C));
+        const dim3 g((unsigned)std::min<size_t>((n + 255) / 256, 152 * 16), 3);
+        k_band_copy<T, TOBAND><<<g, 256, 0, st>>>(bd, src, d.NS, dst, d.NS);
+    }
+    void band_vec_copy(C* dst, const C* src) {  // 3 components of a band spectrum
+        cudaMemcpy2DAsync(dst, d.NS * sizeof(C), src, d.NS * sizeof(C), bd.size * sizeof(C), 3, cudaMemcpyDeviceToDevice,
+                          st);
+    }
+    void stage_run(int kind, T* state, int nin, int nout) {
+        StageArgs<T> a;
+        memset((void*)&a, 0, sizeof(a));
+        for (int i = 0; i < nin; ++i) a.in[i] = pool[B_IN + i];
+        for (int i = 0; i < nout; ++i) a.out[i] = pool[B_OUT + i];
+        a.state = state;
+        a.tw = (const C*)ax[2].tw;
+        a.npts = d.N;
+        a.n2 = d.n2;
+        a.rows = (int)d.rows;
+        a.nb2 = bd.nb2;
+        a.lrb = st_lrb;
+        a.pl = rpl_st;
+        const double bytes =
+            (double)(nin + nout) * bd.nb2 * d.rows * sizeof(C) + (state ? (double)ST_FIELDS * d.N * sizeof(T) : 0.0);
+        constexpr bool f32 = sizeof(T) == 4;
+        PScope ps_(this, kind == 0 ? (f32 ? KC_TANF : KC_TAN64) : (kind == 1 ? (f32 ? KC_ADJF : KC_ADJ64) : KC_SHF), bytes);
+        const size_t units = sizeof(T) == 4 ? (d.rows + 1) / 2 : d.rows;
+        const int grid = (int)((units + (1 << st_lrb) - 1) >> st_lrb);
+        if (!stage_launch(kind, a, grid, st_threads, st_smem, st)) fail(LDDMM_ERR_DEVICE_CHECK);
+    }
+    template <int MODE> void spec_step(C* z0, C* z1, const C* src = nullptr) {
+        StepArgs<T> a;
+        memset((void*)&a, 0, sizeof(a));
+        constexpr int NT = MODE < 2 ? 10 : (MODE < 4 ? 14 : 4);
+        for (int i = 0; i < NT; ++i) a.t[i] = pool[B_SPEC + i];
+        a.e0 = z0;
+        a.x0 = z0 + 3 * d.NS;
+        a.e1 = z1;
+        a.x1 = z1 + 3 * d.NS;
+        a.src = src;
+        a.Lt = Lt;
+        a.Kt = Kt;
+        for (int q = 0; q < 3; ++q) a.dk[q] = tabs.dk[q];
+        a.bd = bd;
+        a.cs = d.NS;
+        a.dt = (T)dt();
+        const int nv = MODE < 4 ? 6 : 3;
+        PScope ps_(this, KC_STEP, (double)bd.size * (sizeof(C) * (NT + (MODE % 2 ? 3 : 2) * nv + (src ? 3 : 0)) + sizeof(T)));
+        k_spec_step<T, MODE><<<(unsigned)((bd.size + 255) / 256), 256, 0, st>>>(a);
+    }
+    // axis-0/1 transforms of a stage's outputs, into the spectra of spec_step
+    void stage_outputs(int nout) {
+        C* o[PLANE_JOBS];
+        for (int i = 0; i < nout; ++i) o[i] = pool[B_SPEC + i];
+        plane_forward(B_OUT, nout, o);
+    }
+    // where the map steps (and the transposed ones) find v_k in the natural layout
+    T* vnat(int k) const { return band_form && exact_grad && band_sweeps ? state(2 * k) + ST_FIELDS * d.N : vss[k % 2]; }
+    T* vstored(int k) const { return band_sweeps ? vnat(k) : state(2 * k); }
+    // One Heun step of the shooting, vhat[0] -> vhat[0], predictor in vhat[1].
+    void band_shoot_step(int k, bool transport, bool kinetic) {
+        const GridI gi{d.n0, d.n1, d.n2};
+        const T ih0 = (T)(1.0 / d.h[0]), ih1 = (T)(1.0 / d.h[1]), ih2 = (T)(1.0 / d.h[2]);
+        for (int stg = 0; stg < 2; ++stg) {
+            C* V = vhat[stg];
+            T* S = state(2 * k + stg);
+            std::vector<BandReq> rq;
+            for (int c = 0; c < 3; ++c) rq.push_back({V + c * d.NS, 0, nullptr, 1.0});
+            rq.push_back({V, 1, nullptr, 1.0});
+            for (int c = 0; c < 3; ++c) rq.push_back({V + c * d.NS, 0, Lt, 1.0});
+            for (int c = 0; c < 3; ++c) rq.push_back({V, 2 + c, Lt, 1.0});
+            plane_inverse(rq, B_IN);
+            if (stg == 0 && transport) {
+                nat_inverse(B_IN, 3, vnat(k));
+                if (k >= 1) {
+                    PScope ps_(this, KC_SL, 12.0 * d.N * sizeof(T));
+                    sl_step(gi, vnat(k - 1), vnat(k), ubuf_at(k - 1), ubuf_at(k), (T)dt(), ih0, ih1, ih2,
+                            prm.interp == LDDMM_INTERP_CUBIC);
+                }
+            }
+            stage_run(2, S, 10, 4);
+            if (stg == 0 && kinetic) dot_async(S + 3 * d.N, S, 3 * d.N, k, d.cell);
+            stage_outputs(4);
+            if (stg == 0) spec_step<4>(vhat[0], vhat[1]);
+            else spec_step<5>(vhat[0], vhat[1]);
+            // the separate Jacobi stages (cross-check) read all 24 fields of V,
+            // which the step has not overwritten in its own stage
+            if (!band_sweeps) {
+                band_copy<false>(stg == 0 ? vhat[0] : vhat[1], tmp);
+                eval_fields({{tmp, 1.0}}, S);
+            }
+        }
+    }
+    void band_tangent_sweep() {
+        for (int k = 0; k < prm.nt; ++k) {
+            ensure_segment(k / cpe);
+            for (int stg = 0; stg < 2; ++stg) {
+                C* Z = tan_[stg];
+                C* X = Z + 3 * d.NS;
+                std::vector<BandReq> rq;
+                for (int c = 0; c < 3; ++c) rq.push_back({Z + c * d.NS, 0, nullptr, 1.0});
+                rq.push_back({Z, 1, nullptr, 1.0});
+                for (int c = 0; c < 3; ++c) rq.push_back({Z + c * d.NS, 0, Lt, 1.0});
+                for (int c = 0; c < 3; ++c) rq.push_back({Z, 2 + c, Lt, 1.0});
+                for (int c = 0; c < 3; ++c) rq.push_back({X + c * d.NS, 0, nullptr, 1.0});
+                rq.push_back({X, 1, nullptr, 1.0});
+                plane_inverse(rq, B_IN);
+                stage_run(0, state(2 * k + stg), 14, 10);
+                stage_outputs(10);
+                if (stg == 0) spec_step<0>(tan_[0], tan_[1]);
+                else spec_step<1>(tan_[0], tan_[1]);
+            }
+        }
+    }
+    void band_adjoint_sweep(const T* eta_src) {
+        for (int k = prm.nt - 1; k >= 0; --k) {
+            ensure_segment(k / cpe);
+            for (int stg = 0; stg < 2; ++stg) {
+                C* Z = adj[stg];
+                C* X = Z + 3 * d.NS;
+                std::vector<BandReq> rq;
+                for (int c = 0; c < 3; ++c) rq.push_back({Z + c * d.NS, 0, Kt, 1.0});
+                rq.push_back({Z, 1, Kt, -1.0});
+                for (int c = 0; c < 3; ++c) rq.push_back({X + c * d.NS, 0, nullptr, 1.0});
+                for (int c = 0; c < 3; ++c) rq.push_back({X, 2 + c, nullptr, 1.0});
+                plane_inverse(rq, B_IN);
+                stage_run(1, state(2 * k + 1 - stg), 10, 14);
+                stage_outputs(14);
+                if (stg == 0) {
+                    spec_step<2>(adj[0], adj[1]);
+                } else {
+                    if (eta_src) band_fwd_vec(eta_src + (size_t)3 * k * d.N, adja);
+                    spec_step<3>(adj[0], adj[1], eta_src ? adja : nullptr);
+                }
+            }
+        }
+    }
+    // tangent sweep's start (eta, xi) = (P dv0, 0); full: dhat keeps F(dv0) for
+    // the regulariser's term
+    void tangent_start(const T* dv0, bool full) {
+        if (band_sweeps && !full) {
+            band_fwd_vec(dv0, tan_[0]);
+        } else {
+            fwd_vec(dv0, dhat);
+            if (band_sweeps) band_copy<true>(dhat, tan_[0]);
+            else mask_copy(dhat, tan_[0]);
+        }
+        cudaMemsetAsync(tan_[0] + 3 * d.NS, 0, 3 * d.NS * sizeof(C), st);
+    }
+    // components first..first + 2 of the tangent sweep's result
+    void tan_to_real(int first, T* out) {
+        if (!band_sweeps) {
+            inv_vec(tan_[prm.nt % 2] + first * d.NS, out, 3, true);
+            return;
+        }
+        std::vector<BandReq> rq;
+        for (int c = 0; c < 3; ++c) rq.push_back({tan_[0] + (first + c) * d.NS, 0, nullptr, 1.0});
+        band_to_real(rq, out);
+    }
+    // P times the adjoint sweep's result (times K with tab)
+    void adj_to_real(T* out, const T* tab = nullptr) {
+        if (!band_sweeps) {
+            spec_to_real2(nullptr, sym(0.0, 0, -1), adj_result(), sym(1.0, 0, -1, 1), out);
+            return;
+        }
+        std::vector<BandReq> rq;
+        for (int c = 0; c < 3; ++c) rq.push_back({adj[0] + c * d.NS, 0, tab, 1.0});
+        band_to_real(rq, out);
+    }
+    // out = w2 L f + P T^T b (metric L2), or K of it: w2 f + K P T^T b.  F(f)
+    // is read where the sum is taken in the spectrum.
+    void assemble(const T* f, const C* fhat, double w2, int space, T* out) {
+        if (!band_sweeps) {
+            if (space == LDDMM_SPACE_V) spec_to_real2(fhat, sym(w2, 0, -1), adj_result(), sym(1.0, -1, -1, 1), out);
+            else spec_to_real2(fhat, sym(w2, 1, -1), adj_result(), sym(1.0, 0, -1, 1), out);
+        } else if (space == LDDMM_SPACE_V) {
+            adj_to_real(out, Kt);
+            PScope ps_(this, KC_MISC, 9.0 * d.N * sizeof(T));
+            k_axpby<T><<<pw_grid(3 * d.N), PW_THREADS, 0, st>>>((T)w2, f, (T)1, out, 3 * d.N);
+        } else {
+            band_copy<false>(adj[0], adja);
+            spec_to_real2(fhat, sym(w2, 1, -1), adja, sym(1.0, 0, -1, 1), out);
+        }
+    }
 
     // spectral out (3) = a_sym . A + b_sym . B  -> real
     void spec_to_real2(const C* A, SymD sa, const C* B, SymD sb, T* out) {
@@ -1675,8 +1952,8 @@ class Engine : public EngineBase {
         int cu = 0;
         for (int k = nt - 1; k >= 0; --k) {
             cudaMemsetAsync(ubar[1 - cu], 0, 3 * d.N * sizeof(T), st);
-            const T* vk = state(2 * k);                            // stage-1 velocity v_k
-            const T* vk1 = k + 1 == nt ? vfin : state(2 * (k + 1));  // v_{k+1}
+            const T* vk = vstored(k);                            // stage-1 velocity v_k
+            const T* vk1 = k + 1 == nt ? vfin : vstored(k + 1);  // v_{k+1}
             {
                 PScope ps_(this, KC_SL, 24.0 * d.N * sizeof(T));
                 T* vb0 = vbar + (size_t)3 * k * d.N;
@@ -1697,18 +1974,14 @@ class Engine : public EngineBase {
     // gradient internals: E into dres[nt+1..nt+3]; gradient real in metric `space`
     void gradient_core(const T* v0, const T* I0, const T* I1, T* grad, int space) {
         NvtxRange nr_("lddmm gradient");
-        shoot_core(v0, true);
+        shoot_core(v0, false);  // no caller reads the kinetic energies
         warp_and_grad(I0);
-        {
-            PScope ps_(this, KC_MISC, 3.0 * d.N * sizeof(T));
-            k_sub<T><<<pw_grid(d.N), PW_THREADS, 0, st>>>(m1, I1, rbuf, d.N);
-        }
-        dot_async(rbuf, nullptr, d.N, prm.nt + 2, d.cell);
-        reg_async(v0, prm.nt + 1);
+        dot_async(m1, I1, d.N, prm.nt + 2, d.cell, true);
+        reg_async(prm.nt + 1);
         if (exact_grad) {
             exact_data_cotangents(I0, I1);
             // eta block from dE/dv_nt, xi block zero; dE/dv_k enter along the way
-            fwd_vec(vbar + (size_t)3 * prm.nt * d.N, adj[0], 1.0, 0, true);
+            band_fwd_vec(vbar + (size_t)3 * prm.nt * d.N, adj[0]);
             cudaMemsetAsync(adj[0] + 3 * d.NS, 0, 3 * d.NS * sizeof(C), st);
             adjoint_sweep(vbar);
         } else {
@@ -1716,16 +1989,13 @@ class Engine : public EngineBase {
                 PScope ps_(this, KC_MISC, 8.0 * d.N * sizeof(T));
                 k_final_source<T><<<pw_grid(d.N), PW_THREADS, 0, st>>>(m1, I1, gm1, nullptr, rs, 0, d.N);
             }
-            fwd_vec(rs, adj[0] + 3 * d.NS, 1.0, 0, true);
+            band_fwd_vec(rs, adj[0] + 3 * d.NS);
             cudaMemsetAsync(adj[0], 0, 3 * d.NS * sizeof(C), st);
             adjoint_sweep();
         }
         // g_L2 = 2 w L v0 + T^T b ;  V: K g_L2 = 2 w v0 + K T^T b
         const double w2 = 2.0 * prm.weight;
-        if (space == LDDMM_SPACE_V)
-            spec_to_real2(v0full, sym(w2, 0, -1), adj_result(), sym(1.0, -1, -1, 1), grad);
-        else
-            spec_to_real2(v0full, sym(w2, 1, -1), adj_result(), sym(1.0, 0, -1, 1), grad);
+        assemble(v0, v0full, w2, space, grad);
         lin_valid = true;
     }
     // ---- the Hessian-vector product as a CUDA graph.  Its ~220 launches
@@ -1777,25 +2047,21 @@ class Engine : public EngineBase {
 
     void hessvec_core(const T* dv0, T* out, int space) {
         NvtxRange nr_("lddmm hessvec");
-        fwd_vec(dv0, dhat);
-        mask_copy(dhat, tan_[0]);
-        cudaMemsetAsync(tan_[0] + 3 * d.NS, 0, 3 * d.NS * sizeof(C), st);
+        // the metric L2 adds 2 w L dv0, which needs the whole spectrum of dv0
+        tangent_start(dv0, space == LDDMM_SPACE_L2);
         tangent_sweep();
         T* xi = rs;
-        inv_vec(tan_[prm.nt % 2] + 3 * d.NS, xi, 3, true);
+        tan_to_real(3, xi);
         T* c = rs + 3 * d.N;
         {
             PScope ps_(this, KC_MISC, 8.0 * d.N * sizeof(T));
             k_final_source<T><<<pw_grid(d.N), PW_THREADS, 0, st>>>(m1, nullptr, gm1, xi, c, 1, d.N);
         }
-        fwd_vec(c, adj[0] + 3 * d.NS, 1.0, 0, true);
+        band_fwd_vec(c, adj[0] + 3 * d.NS);
         cudaMemsetAsync(adj[0], 0, 3 * d.NS * sizeof(C), st);
         adjoint_sweep();
         const double w2 = 2.0 * prm.weight;
-        if (space == LDDMM_SPACE_V)
-            spec_to_real2(dhat, sym(w2, 0, -1), adj_result(), sym(1.0, -1, -1, 1), out);
-        else
-            spec_to_real2(dhat, sym(w2, 1, -1), adj_result(), sym(1.0, 0, -1, 1), out);
+        assemble(dv0, dhat, w2, space, out);
     }
 
     // ------------------------------------------------------------ ABI operations
@@ -1851,12 +2117,10 @@ class Engine : public EngineBase {
         if (!dv0) return fail(LDDMM_ERR_ARG);
         if (!lin_valid) return LDDMM_ERR_NOT_LINEARIZED;
         scan_inputs({{dv0, 3 * d.N}});
-        fwd_vec((const T*)dv0, dhat);
-        mask_copy(dhat, tan_[0]);
-        cudaMemsetAsync(tan_[0] + 3 * d.NS, 0, 3 * d.NS * sizeof(C), st);
+        tangent_start((const T*)dv0, false);
         tangent_sweep();
-        if (eta1) inv_vec(tan_[prm.nt % 2], (T*)eta1, 3, true);
-        if (xi1) inv_vec(tan_[prm.nt % 2] + 3 * d.NS, (T*)xi1, 3, true);
+        if (eta1) tan_to_real(0, (T*)eta1);
+        if (xi1) tan_to_real(3, (T*)xi1);
         return finish();
     }
 
@@ -1865,11 +2129,11 @@ class Engine : public EngineBase {
         if (!bxi || !out) return fail(LDDMM_ERR_ARG);
         if (!lin_valid) return LDDMM_ERR_NOT_LINEARIZED;
         scan_inputs({{beta, 3 * d.N}, {bxi, 3 * d.N}});
-        fwd_vec((const T*)bxi, adj[0] + 3 * d.NS, 1.0, 0, true);
-        if (beta) fwd_vec((const T*)beta, adj[0], 1.0, 0, true);
+        band_fwd_vec((const T*)bxi, adj[0] + 3 * d.NS);
+        if (beta) band_fwd_vec((const T*)beta, adj[0]);
         else cudaMemsetAsync(adj[0], 0, 3 * d.NS * sizeof(C), st);
         adjoint_sweep();
-        spec_to_real2(nullptr, sym(0.0, 0, -1), adj_result(), sym(1.0, 0, -1, 1), (T*)out);
+        adj_to_real((T*)out);
         return finish();
     }
 
@@ -1936,10 +2200,10 @@ class Engine : public EngineBase {
             PScope ps_(this, KC_MISC, 8.0 * d.N * sizeof(T));
             k_vjp_source<T><<<pw_grid(d.N), PW_THREADS, 0, st>>>((const T*)G, gm1, rs, d.N);
         }
-        fwd_vec(rs, adj[0] + 3 * d.NS, 1.0, 0, true);
+        band_fwd_vec(rs, adj[0] + 3 * d.NS);
         cudaMemsetAsync(adj[0], 0, 3 * d.NS * sizeof(C), st);
         adjoint_sweep();
-        spec_to_real2(nullptr, sym(0.0, 0, -1), adj_result(), sym(1.0, 0, -1, 1), (T*)out);
+        adj_to_real((T*)out);
         return finish();
     }
 
@@ -1950,7 +2214,7 @@ class Engine : public EngineBase {
 
     // ------------------------------------------------------------ GN-Krylov
     double energy_at(const T* v, const T* I0, const T* I1) {
-        shoot_core(v, true);
+        shoot_core(v, false);
         lin_valid = false;
         const GridI gi{d.n0, d.n1, d.n2};
         {
@@ -1958,12 +2222,8 @@ class Engine : public EngineBase {
             k_warp<T><<<pw_grid(d.N), PW_THREADS, 0, st>>>(gi, I0, u1(), m1, (T)(1.0 / d.h[0]), (T)(1.0 / d.h[1]),
                                                           (T)(1.0 / d.h[2]), prm.interp == LDDMM_INTERP_CUBIC, d.N);
         }
-        {
-            PScope ps_(this, KC_MISC, 3.0 * d.N * sizeof(T));
-            k_sub<T><<<pw_grid(d.N), PW_THREADS, 0, st>>>(m1, I1, rbuf, d.N);
-        }
-        dot_async(rbuf, nullptr, d.N, prm.nt + 2, d.cell);
-        reg_async(v, prm.nt + 1);
+        dot_async(m1, I1, d.N, prm.nt + 2, d.cell, true);
+        reg_async(prm.nt + 1);
         if (fetch(0, prm.nt + 3) != LDDMM_OK) return NAN;
         return hres[prm.nt + 2] + prm.weight * hres[prm.nt + 1];
     }
@@ -2131,11 +2391,7 @@ class Engine : public EngineBase {
         minmax_async(gsp, n3, 60);
         if (fetch(60, 1) != LDDMM_OK) return status;
         R.gnorm_rel = g0max > 0 ? hres[60] / g0max : 0.0;
-        {
-            PScope ps_(this, KC_MISC, 3.0 * d.N * sizeof(T));
-            k_sub<T><<<pw_grid(d.N), PW_THREADS, 0, st>>>(I0, I1, rbuf, d.N);
-        }
-        const double d0 = dot_now(rbuf, nullptr, d.N);
+        const double d0 = dot_now(I0, I1, d.N, true);
         R.mse_rel = d0 > 0 ? data / d0 : 0.0;
         T* J = rs + 9 * d.N;
         jacdet_into(u1(), J);

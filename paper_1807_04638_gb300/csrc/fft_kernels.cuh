@@ -239,7 +239,7 @@ __global__ void __launch_bounds__(FFT_THREADS) k_pass_axis2(const __grid_constan
         for (int e = threadIdx.x; e < 2 * TL * n2h; e += blockDim.x) {
             const int row = e % (2 * TL), k = e / (2 * TL);
             cpx<T> acc = mk((T)0, (T)0);
-            if (row < nr)
+            if (row < nr && k < pp.nb2)  // planes above the band are zero
                 for (int b = 0; b < job.nin; ++b)
                     acc = acc + job.isym[b].scale * ((const cpx<T>*)job.in[b])[(size_t)k * rows + r0 + row];
             H[row * Ph + k] = acc;
@@ -303,7 +303,7 @@ __global__ void __launch_bounds__(FFT_THREADS) k_pass_axis2(const __grid_constan
             __syncthreads();
         }
         cpx<T>* out = (cpx<T>*)job.out[0];
-        for (int e = threadIdx.x; e < 2 * TL * n2h; e += blockDim.x) {
+        for (int e = threadIdx.x; e < 2 * TL * pp.nb2; e += blockDim.x) {
             const int row = e % (2 * TL), k = e / (2 * TL);
             if (row < nr) out[(size_t)k * rows + r0 + row] = H[row * Ph + k];
         }

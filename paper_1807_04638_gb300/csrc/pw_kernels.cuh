@@ -581,13 +581,95 @@ __device__ __forceinline__ double block_reduce(double v, int op) {
     return v;
 }
 
-// partial[b] = sum over this block's share of a[x]*b[x] (b == nullptr: a[x]^2)
-template <class T>
+// 16-byte loads of an array that may start anywhere: V elements at a time from
+// its first 16-byte boundary, the few before and after it one by one.  A
+// reduction that reads one element per thread and step is bound by the latency
+// of its loads (0.9 TB/s at 3 x 128^3 FP32); four 16-byte loads in flight per
+// thread bring it to the rate of its FP64 adds or of memory.
+template <class T> struct Vec16 {
+    static constexpr int V = 16 / (int)sizeof(T);
+    T v[V];
+};
+__device__ __forceinline__ Vec16<float> ld16(const float* p) {
+    const float4 q = __ldg((const float4*)p);
+    return {{q.x, q.y, q.z, q.w}};
+}
+__device__ __forceinline__ Vec16<double> ld16(const double* p) {
+    const double2 q = __ldg((const double2*)p);
+    return {{q.x, q.y}};
+}
+// elements of a before its first 16-byte boundary (at most n)
+template <class T> __device__ __forceinline__ size_t head16(const T* a, size_t n) {
+    const size_t h = ((16 - ((size_t)a & 15)) & 15) / sizeof(T);
+    return h < n ? h : n;
+}
+
+// what a dot product sums: a b, a^2, or (a - b)^2
+enum { DOT_AB = 0, DOT_AA = 1, DOT_DIFF = 2 };
+template <class T, int KIND> __device__ __forceinline__ double dot_term(T a, T b) {
+    if (KIND == DOT_AB) return (double)a * (double)b;
+    const double x = KIND == DOT_AA ? (double)a : (double)(a - b);
+    return x * x;
+}
+// partial[block] = sum over this block's share of the terms
+template <class T, int KIND>
 __global__ void k_dot_partial(const T* __restrict__ a, const T* __restrict__ b, size_t n, double* __restrict__ partial) {
+    constexpr int V = Vec16<T>::V, U = 4;
+    const size_t id = blockIdx.x * (size_t)blockDim.x + threadIdx.x, step = (size_t)gridDim.x * blockDim.x;
+    double acc[U] = {0.0, 0.0, 0.0, 0.0};
+    size_t done = 0;
+    if (KIND == DOT_AA || (((size_t)a ^ (size_t)b) & 15) == 0) {
+        const size_t h = head16(a, n), nv = (n - h) / V;
+        if (id < h) acc[0] += dot_term<T, KIND>(a[id], KIND == DOT_AA ? (T)0 : b[id]);
+        for (size_t q = id; q < nv; q += U * step) {
+            Vec16<T> x[U], y[U];
+#pragma unroll
+            for (int u = 0; u < U; ++u) {
+                const size_t i = q + u * step;
+                if (i < nv) {
+                    x[u] = ld16(a + h + i * V);
+                    if (KIND != DOT_AA) y[u] = ld16(b + h + i * V);
+                }
+            }
+#pragma unroll
+            for (int u = 0; u < U; ++u)
+                if (q + u * step < nv) {
+#pragma unroll
+                    for (int e = 0; e < V; ++e) acc[u] += dot_term<T, KIND>(x[u].v[e], KIND == DOT_AA ? (T)0 : y[u].v[e]);
+                }
+        }
+        done = h + nv * V;
+    }
+    for (size_t x = done + id; x < n; x += step) acc[0] += dot_term<T, KIND>(a[x], KIND == DOT_AA ? (T)0 : b[x]);
+    const double s = block_reduce((acc[0] + acc[1]) + (acc[2] + acc[3]), 0);
+    if (threadIdx.x == 0) partial[blockIdx.x] = s;
+}
+
+// partial[block] = sum over the half spectrum F(v) [k2][k0][k1] of three
+// components (stride cs) of L |F(v)|^2, entries with a conjugate partner
+// twice: N <L v, v> by Parseval's identity
+template <class T>
+__global__ void k_spec_energy(const cpx<T>* __restrict__ vh, size_t cs, SpecTabs<T> tb, int n0, int n1, int n2h,
+                              double* __restrict__ partial) {
     double acc = 0.0;
-    for (size_t x = blockIdx.x * (size_t)blockDim.x + threadIdx.x; x < n; x += (size_t)gridDim.x * blockDim.x) {
-        const double av = (double)a[x];
-        acc += av * (b ? (double)b[x] : av);
+    const int rows = n0 * n2h;
+    for (int r = blockIdx.x; r < rows; r += gridDim.x) {
+        const int k2 = r / n0, k0 = r - k2 * n0;
+        const double w = k2 == 0 || 2 * k2 == tb.n[2] ? 1.0 : 2.0;
+        const T q = tb.ksq[0][k0] + tb.ksq[2][k2];
+        for (int k1 = threadIdx.x; k1 < n1; k1 += blockDim.x) {
+            const T base = (T)1 + tb.alpha * (q + tb.ksq[1][k1]);
+            T L = (T)1;
+            for (int e = 0; e < tb.s; ++e) L *= base;
+            const size_t x = (size_t)r * n1 + k1;
+            double m = 0.0;
+#pragma unroll
+            for (int c = 0; c < 3; ++c) {
+                const cpx<T> z = vh[c * cs + x];
+                m += (double)z.x * (double)z.x + (double)z.y * (double)z.y;
+            }
+            acc += w * (double)L * m;
+        }
     }
     acc = block_reduce(acc, 0);
     if (threadIdx.x == 0) partial[blockIdx.x] = acc;
@@ -626,10 +708,27 @@ template <class T> struct ScanArgs {
 template <class T>
 __global__ void k_nonfinite_scan(const __grid_constant__ ScanArgs<T> a, double* __restrict__ flag) {
     bool bad = false;
-    const size_t stride = (size_t)gridDim.x * blockDim.x;
-    for (int i = 0; i < a.cnt; ++i)
-        for (size_t x = blockIdx.x * (size_t)blockDim.x + threadIdx.x; x < a.n[i]; x += stride)
-            bad |= !isfinite(a.p[i][x]);
+    constexpr int V = Vec16<T>::V, U = 4;
+    const size_t id = blockIdx.x * (size_t)blockDim.x + threadIdx.x, step = (size_t)gridDim.x * blockDim.x;
+    for (int k = 0; k < a.cnt; ++k) {
+        const T* const p = a.p[k];
+        const size_t n = a.n[k], h = head16(p, n), nv = (n - h) / V;
+        if (id < h) bad |= !isfinite(p[id]);
+        for (size_t q = id; q < nv; q += U * step) {
+            Vec16<T> x[U];
+#pragma unroll
+            for (int u = 0; u < U; ++u) {
+                const size_t i = q + u * step;
+                if (i < nv) x[u] = ld16(p + h + i * V);
+                else x[u] = Vec16<T>{};
+            }
+#pragma unroll
+            for (int u = 0; u < U; ++u)
+#pragma unroll
+                for (int e = 0; e < V; ++e) bad |= !isfinite(x[u].v[e]);
+        }
+        for (size_t x = h + nv * V + id; x < n; x += step) bad |= !isfinite(p[x]);
+    }
     if (__syncthreads_or(bad) && threadIdx.x == 0) *flag = 1.0;
 }
 
@@ -685,13 +784,6 @@ __global__ void k_vjp_source(const T* __restrict__ G, const T* __restrict__ gm, 
         out[N + x] = g * gm[N + x];
         out[2 * N + x] = g * gm[2 * N + x];
     }
-}
-
-// r = m1 - I1
-template <class T>
-__global__ void k_sub(const T* __restrict__ a, const T* __restrict__ b, T* __restrict__ r, size_t n) {
-    for (size_t i = blockIdx.x * (size_t)blockDim.x + threadIdx.x; i < n; i += (size_t)gridDim.x * blockDim.x)
-        r[i] = a[i] - b[i];
 }
 
 // det(I + Du), Du[c][j] = D_j u_c at field 3c + j
