@@ -105,9 +105,14 @@ static lddmm_status noalloc_run(const Dims& d, double alpha, int s, int power, c
     for (int a = 0; a < 3; ++a) tw[a] = (C*)carve(ns[a] * sizeof(C));
     for (int a = 0; a < 3; ++a) dk[a] = (T*)carve(nk[a] * sizeof(T));
     for (int a = 0; a < 3; ++a) ks[a] = (T*)carve(nk[a] * sizeof(T));
-    C* A = (C*)carve(d.NS * sizeof(C));
-    C* B = (C*)carve(d.NS * sizeof(C));
-    if (off > NOALLOC_SCRATCH_BYTES) return LDDMM_ERR_TOO_LARGE;
+    // as many components at a time as the rest of the scratch holds (two half
+    // spectra each): a small grid is bound by its launches
+    const size_t field = (d.NS * sizeof(C) + 255) & ~(size_t)255;
+    off = (off + 255) & ~(size_t)255;
+    if (off + 2 * field > NOALLOC_SCRATCH_BYTES) return LDDMM_ERR_TOO_LARGE;
+    const int group = (int)std::min<size_t>(std::min<size_t>((NOALLOC_SCRATCH_BYTES - off) / (2 * field), MAXJOBS), ncomp);
+    C* const A = (C*)((unsigned char*)base + off);
+    C* const B = (C*)((unsigned char*)A + group * field);
 
     k_noalloc_tables<T><<<4, 128, 0, st>>>(d.n0, d.n1, d.n2, d.len[0], d.len[1], d.len[2], tw[0], tw[1], tw[2], dk[0],
                                           dk[1], dk[2], ks[0], ks[1], ks[2]);
@@ -136,18 +141,22 @@ static lddmm_status noalloc_run(const Dims& d, double alpha, int s, int power, c
     int TL2 = 16;
     while (TL2 > 1 && ((size_t)2 * TL2 * Ph2 + 2 * TL2 * P2) * sizeof(C) > budget) TL2 /= 2;
     const size_t sm2 = ((size_t)2 * TL2 * Ph2 + 2 * TL2 * P2) * sizeof(C);
-    bool fast[3];
+    bool fast[3], gen[3] = {false, false, false};
+    RPlan gpl[2];
     for (int a = 0; a < 3; ++a) {
         PassParams<T> dummy;
         const bool aligned = a != 0 || sizeof(T) == 8 || ns[1] % 2 == 0;
         fast[a] = FastPass<T>::has(ns[a]) && aligned && !force_generic_fft() &&
                   FastPass<T>::launch(ns[a], a, 0, dummy, 0, 0, 0, 0, 0, st, true);
     }
+    for (int a = 0; a < 2; ++a)
+        if (!fast[a] && !force_generic_fft() && (gpl[a] = radix_plan3(ns[a])).n) gen[a] = GenPass<T>::prepare(a, gpl[a]);
     if (!raise_smem_limit(k_pass_c2c<T, 0>, smc[0]) || !raise_smem_limit(k_pass_c2c<T, 1>, smc[1]) ||
         !raise_smem_limit(k_pass_axis2<T>, sm2))
         return LDDMM_ERR_CUDA;
 
-    auto one = [&](int axis, int sign, const void* src, void* dst, SymD sy) {
+    // nc transforms of one axis: fields at src and dst with byte strides ss and ds
+    auto pass = [&](int axis, int sign, int nc, const void* src, size_t ss, void* dst, size_t ds, SymD sy) {
         PassParams<T> pp;
         memset(&pp, 0, sizeof(pp));
         pp.ax.n = ns[axis];
@@ -160,38 +169,41 @@ static lddmm_status noalloc_run(const Dims& d, double alpha, int s, int power, c
         pp.sign = sign;
         full_band(pp);
         pp.tabs = tabs;
-        pp.njobs = 1;
-        PassJobT<T>& j = pp.jobs[0];
-        j.nin = 1;
-        j.in[0] = src;
-        j.nout = 1;
-        j.out[0] = dst;
+        pp.njobs = nc;
         SymT<T> unit;
         unit.scale = (T)1;
         unit.lpow = 0;
         unit.deriv = -1;
         unit.mask = 0;
         const SymT<T> syt = to_symt<T>(sy);
-        j.isym[0] = sign > 0 ? unit : syt;
-        j.osym[0] = sign > 0 ? syt : unit;
+        for (int c = 0; c < nc; ++c) {
+            PassJobT<T>& j = pp.jobs[c];
+            j.nin = j.nout = 1;
+            j.in[0] = (const unsigned char*)src + c * ss;
+            j.out[0] = (unsigned char*)dst + c * ds;
+            j.isym[0] = sign > 0 ? unit : syt;
+            j.osym[0] = sign > 0 ? syt : unit;
+        }
         if (fast[axis]) {
-            FastPass<T>::launch(ns[axis], axis, sign, pp, 1, d.rows, d.n0, d.n1, d.n2h, st);
+            FastPass<T>::launch(ns[axis], axis, sign, pp, nc, d.rows, d.n0, d.n1, d.n2h, st);
+        } else if (gen[axis]) {
+            GenPass<T>::launch(axis, sign, pp, nc, gpl[axis], st);
         } else if (axis == 2) {
             pp.TL = TL2;
             pp.P = P2;
             pp.Ph = Ph2;
             const int gx = (int)((d.rows + 2 * TL2 - 1) / (2 * TL2));
-            k_pass_axis2<T><<<dim3(gx, 1), FFT_THREADS, sm2, st>>>(pp);
+            k_pass_axis2<T><<<dim3(gx, nc), FFT_THREADS, sm2, st>>>(pp);
         } else if (axis == 1) {
             pp.TL = TLc[1];
             pp.P = Pc[1];
             const int gx = (int)(((size_t)d.n2h * d.n0 + TLc[1] - 1) / TLc[1]);
-            k_pass_c2c<T, 1><<<dim3(gx, 1), FFT_THREADS, smc[1], st>>>(pp);
+            k_pass_c2c<T, 1><<<dim3(gx, nc), FFT_THREADS, smc[1], st>>>(pp);
         } else {
             pp.TL = TLc[0];
             pp.P = Pc[0];
             const int gx = d.n2h * ((d.n1 + TLc[0] - 1) / TLc[0]);
-            k_pass_c2c<T, 0><<<dim3(gx, 1), FFT_THREADS, smc[0], st>>>(pp);
+            k_pass_c2c<T, 0><<<dim3(gx, nc), FFT_THREADS, smc[0], st>>>(pp);
         }
     };
     SymD unit;
@@ -203,15 +215,15 @@ static lddmm_status noalloc_run(const Dims& d, double alpha, int s, int power, c
     lp.lpow = power;
     SymD inv = unit;
     inv.scale = 1.0 / (double)d.N;
-    for (int c = 0; c < ncomp; ++c) {
-        const T* x = in + (size_t)c * d.N;
-        T* y = out + (size_t)c * d.N;
-        one(2, -1, x, A, unit);  // rows -> [k2][row]
-        one(1, -1, A, B, unit);
-        one(0, -1, B, A, lp);    // full spectrum times L_hat^power
-        one(0, +1, A, B, inv);   // 1/N normalisation of the inverse
-        one(1, +1, B, A, unit);
-        one(2, +1, A, y, unit);
+    const size_t real = d.N * sizeof(T);
+    for (int c = 0; c < ncomp; c += group) {
+        const int nc = std::min(group, ncomp - c);
+        pass(2, -1, nc, in + (size_t)c * d.N, real, A, field, unit);  // rows -> [k2][row]
+        pass(1, -1, nc, A, field, B, field, unit);
+        pass(0, -1, nc, B, field, A, field, lp);   // full spectrum times L_hat^power
+        pass(0, +1, nc, A, field, B, field, inv);  // 1/N normalisation of the inverse
+        pass(1, +1, nc, B, field, A, field, unit);
+        pass(2, +1, nc, A, field, out + (size_t)c * d.N, real, unit);
     }
     return cudaGetLastError() == cudaSuccess ? LDDMM_OK : LDDMM_ERR_CUDA;
 }
