@@ -1772,7 +1772,7 @@ class Engine : public EngineBase {
         a.dt = (T)dt();
         const int nv = MODE < 4 ? 6 : 3;
         PScope ps_(this, KC_STEP, (double)bd.size * (sizeof(C) * (NT + (MODE % 2 ? 3 : 2) * nv + (src ? 3 : 0)) + sizeof(T)));
-        k_spec_step<T, MODE><<<(unsigned)((bd.size + 255) / 256), 256, 0, st>>>(a);
+        launch_dependent(k_spec_step<T, MODE>, dim3((unsigned)((bd.size + 255) / 256)), 256, 0, st, a);
     }
     // axis-0/1 transforms of a stage's outputs, into the spectra of spec_step
     void stage_outputs(int nout) {

@@ -55,4 +55,30 @@ inline int persistent_grid(int items, int per_sm = 3) {
     return std::max(1, std::min(items, per_sm * sms));
 }
 
+// Launch that may begin before the kernel in front of it on the stream has
+// ended (programmatic dependent launch): the kernel's prologue overlaps the
+// other's last blocks.  Every kernel launched this way calls after_previous()
+// before its first access to memory that another kernel of the stream writes
+// or reads, and dependents_may_launch() when it is about to write its last
+// results: at that point the launch latency and the prologue are hidden and
+// the dependents take no room from its own blocks.  Hessian-vector product at
+// 64^3: 1.52 ms without, 1.42 ms so, 1.64 ms with the call at the kernel's
+// start; at 128^3 7.11, 6.97 and 6.91 ms.
+template <class A>
+inline void launch_dependent(void (*kernel)(A), dim3 grid, unsigned threads, size_t smem, cudaStream_t st, const A& a) {
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = grid;
+    cfg.blockDim = dim3(threads);
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = st;
+    cudaLaunchAttribute at[1];
+    at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    at[0].val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = at;
+    cfg.numAttrs = 1;
+    cudaLaunchKernelEx(&cfg, kernel, a);
+}
+__device__ __forceinline__ void after_previous() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+__device__ __forceinline__ void dependents_may_launch() { asm volatile("griddepcontrol.launch_dependents;"); }
+
 }  // namespace lddmm

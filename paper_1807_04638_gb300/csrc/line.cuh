@@ -62,6 +62,7 @@ __global__ void __launch_bounds__(line_threads(N), 512 / line_threads(N)) k_line
     const bool on = l0 < lines;
     const int b0p = bd.b0p, n1 = AXIS == 1 ? N : bd.n1;
     C2* const buf = bufs + c;
+    after_previous();
     __syncthreads();
 
     // ---- stage 0: element n = j + r M of the line
@@ -81,7 +82,7 @@ __global__ void __launch_bounds__(line_threads(N), 512 / line_threads(N)) k_line
                 if (job.kind == 0) {
 #pragma unroll
                     for (int r = 0; r < AA; ++r) {
-                        const int k1 = j + r * M, c1 = LineBand<N>::template at<M>(j, r);
+                        const int c1 = LineBand<N>::template at<M>(j, r);
                         if (c1 >= 0) v[r] = pair(__ldg((const float4*)(job.in + o0 + (unsigned)(c1 * b0p))));
                     }
                 } else {
@@ -115,9 +116,8 @@ __global__ void __launch_bounds__(line_threads(N), 512 / line_threads(N)) k_line
                 }
 #pragma unroll
                 for (int r = 0; r < AA; ++r) {
-                    const int k1 = j + r * M, c1 = LineBand<N>::template at<M>(j, r);
+                    const int c1 = LineBand<N>::template at<M>(j, r);
                     if (c1 < 0) continue;
-                    (void)k1;
                     P2 f = sc;
                     if (tab) {
                         const float2 t = __ldg((const float2*)(tab + o0 + (unsigned)(c1 * b0p)));
@@ -180,6 +180,7 @@ __global__ void __launch_bounds__(line_threads(N), 512 / line_threads(N)) k_line
         }
         __syncthreads();
     }
+    dependents_may_launch();
     // ---- last stage: output k = i + r ML
     constexpr int ML = N / CC;
     if (!on) return;

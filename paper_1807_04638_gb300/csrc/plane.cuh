@@ -16,6 +16,7 @@
 // axes as two launches (PH = 1, then 2; forward 2, then 1) over column and line
 // tiles with the half-transformed band [k2][i1][k0c] between them.
 #pragma once
+#include "launch_util.cuh"
 #include "radix.cuh"
 
 namespace lddmm {
@@ -98,6 +99,8 @@ template <class T> struct StepArgs {
 template <class T, int MODE>
 __global__ void __launch_bounds__(256) k_spec_step(const __grid_constant__ StepArgs<T> a) {
     const Band& bd = a.bd;
+    dependents_may_launch();
+    after_previous();
     const int i = blockIdx.x * 256 + threadIdx.x;
     if (i >= (int)bd.size) return;
     const int q = i / bd.b0p, kc0 = min(i - q * bd.b0p, bd.b0 - 1), k2 = q / bd.b1, kc1 = q - k2 * bd.b1;

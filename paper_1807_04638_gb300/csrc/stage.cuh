@@ -37,6 +37,7 @@
 #pragma once
 #include <type_traits>
 
+#include "launch_util.cuh"
 #include "radix.cuh"
 
 namespace lddmm {
@@ -433,6 +434,7 @@ __global__ void __launch_bounds__(STAGE_THREADS) k_stage(const __grid_constant__
         const int o1 = KIND == 0 ? (ph == 0 ? 5 : 2) : (KIND == 1 ? (ph == 0 ? 5 : 7) : 2);
 #pragma unroll 1
         for (int o = o0; o < o1; ++o) {
+            if (ph == PHASES - 1 && o == o1 - 1) dependents_may_launch();
             int which = o;  // 0 / 1: (A_0, A_1) / (A_2, A_3)
             if constexpr (KIND == 1) which = o >= 5 ? o - 5 : o + 2;
             switch (which) {
@@ -608,6 +610,7 @@ __global__ void __launch_bounds__(NN ? (NN / P * stage_rb(NN, P) + 31) / 32 * 32
     };
     // the next inverse line of the block after l (-1: none)
     auto next_line = [&](int l) { return KIND == 0 ? (l == 6 ? 0 : (l == 4 ? -1 : l + 1)) : (l == 4 ? -1 : l + 1); };
+    after_previous();
     issue(KIND == 0 ? 5 : 0, 0);
 
     auto inv = [&](int l, P2(&u)[P], P2(&w)[P]) {
@@ -951,6 +954,7 @@ __global__ void __launch_bounds__(NN ? (NN / P * stage_rb(NN, P) + 31) / 32 * 32
         const int o1 = KIND == 0 ? (ph == 0 ? 5 : 2) : (KIND == 1 ? (ph == 0 ? 5 : 7) : 2);
 #pragma unroll 1
         for (int o = o0; o < o1; ++o) {
+            if (ph == PHASES - 1 && o == o1 - 1) dependents_may_launch();
             int which = o;  // 0 / 1: (A_0, A_1) / (A_2, A_3)
             if constexpr (KIND == 1) which = o >= 5 ? o - 5 : o + 2;
             switch (which) {
@@ -1044,7 +1048,8 @@ inline bool stage_go(K kernel, const A& a, int grid, int threads, size_t smem, c
         cudaGetLastError();
         return false;
     }
-    kernel<<<grid, threads, smem, st>>>(a);
+    if constexpr (sizeof(a.tw->x) == 4) launch_dependent(kernel, dim3(grid), threads, smem, st, a);
+    else kernel<<<grid, threads, smem, st>>>(a);
     return true;
 }
 

@@ -52,7 +52,7 @@ template <int MODE> static bool line_go(const PlaneArgs<float>& a, dim3 grid, cu
         cudaGetLastError();
         return false;
     }
-    k<<<grid, line_threads(N), line_smem(N), st>>>(a);
+    launch_dependent(k, grid, line_threads(N), line_smem(N), st, a);
     return true;
 }
 template <>
