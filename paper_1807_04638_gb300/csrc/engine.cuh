@@ -165,13 +165,14 @@ inline Layout layout_for(const Dims& d, const lddmm_params* p, size_t tsize) {
     Layout L;
     // pool + vhat(6) + v0hat(3) + v0full(3) + R1(3) + tan(12) + tb(6) + adj(12) + adja(6) + dhat(3) + tmp(3)
     L.spec_fields = POOL + 6 + 3 + 3 + 3 + 12 + 6 + 12 + 6 + 3 + 3;
-    // vfin(6) + u(6) + scratch + m1(1) + gm1(3) + PCG (x r z p q g vt: 21)
-    // + FP32 copies of the last two stage-1 velocities for the map transport (6)
+    // vfin(6) + scratch + m1(1) + gm1(3) + PCG (x r z p q g vt: 21); for the map
+    // transport u(6) and the last two stage-1 velocities (6), in FP32 one of
+    // each (6) and both of each with four numbers a point (16)
     const bool bf16 = p->state_dtype == LDDMM_BF16;
     const int cpe = p->checkpoint_every <= 1 ? p->nt : std::min(p->checkpoint_every, p->nt);
     const bool ckpt = cpe < p->nt;
     const int nseg = (p->nt + cpe - 1) / cpe;
-    L.real_fields = 6 + 6 + RSCR + 1 + 3 + 21 + 6;
+    L.real_fields = 6 + RSCR + 1 + 3 + 21 + (tsize == 4 ? 22 : 12);
     // exact discrete gradient: every map u_k, every dE/dv_k, two dE/du buffers
     if (p->gradient_mode == LDDMM_GRAD_DISCRETE) L.real_fields += (size_t)6 * (p->nt + 1) + 6;
     if (ckpt) L.spec_fields += (size_t)3 * nseg;  // spectral v at the checkpoints
@@ -192,9 +193,9 @@ inline bool force_generic_fft() {
     const char* e = getenv("LDDMM_GENERIC_FFT");
     return e && e[0] == '1';
 }
-// LDDMM_SL_GATHER=1 makes the FP32 map steps use the global-gather kernel
-// k_sl_step instead of the shared-memory staged one; used to cross-check the
-// staged kernel, including its fallback for stencils that leave the box.
+// LDDMM_SL_GATHER=1 makes the FP32 map steps gather every point from global
+// memory instead of the staged box; used to cross-check the staged taps,
+// including the fallback for stencils that leave the box.
 inline bool force_sl_gather() {
     const char* e = getenv("LDDMM_SL_GATHER");
     return e && e[0] == '1';
@@ -320,6 +321,7 @@ class Engine : public EngineBase {
     bool ckpt = false;
     C* cps = nullptr;
     T *vfin, *ubuf[2], *rs, *m1, *gm1, *vss[2] = {nullptr, nullptr};
+    float4* sl4[4] = {nullptr, nullptr, nullptr, nullptr};  // FP32 map steps: v (2), u (2), one float4 a point
     // exact discrete gradient: maps u_k (k = 0..nt), dE/dv_k, dE/du ping-pong
     T *ustore = nullptr, *vbar = nullptr, *ubar[2] = {nullptr, nullptr};
     bool exact_grad = false;
@@ -335,7 +337,7 @@ class Engine : public EngineBase {
     RPlan gpl[2];
     // band-limited transforms (all three passes register-blocked, dealiasing on)
     bool band_ok = false;
-    bool sl_staged = false;  // FP32 map steps use k_sl_step_staged
+    bool sl_plain = false;  // FP32 map steps by the plain loops (cross-check)
     bool fused = false;      // FP32 Jacobi stages use k_fused_stage
     int bnb2 = 0, bc1 = 0, bs1 = 0;
     // band form (plane.cuh, stage.cuh): dealiasing on, states in the compute type
@@ -493,10 +495,12 @@ class Engine : public EngineBase {
         const size_t nstate = (size_t)2 * (ckpt ? cpe : prm.nt) * 24 * d.N;
         if (bf16) states = carve<__nv_bfloat16>(nstate);
         else states = carve<T>(nstate);
-        for (int i = 0; i < 2; ++i) vss[i] = carve<T>(3 * d.N);
+        constexpr int two = sizeof(T) == 4 ? 1 : 2;  // FP32 keeps the last step's fields in sl4
+        for (int i = 0; i < 2; ++i) vss[i] = i < two ? carve<T>(3 * d.N) : vss[0];
+        for (int i = 0; i < 4 && sizeof(T) == 4; ++i) sl4[i] = carve<float4>(d.N);
         if (ckpt) cps = carve<C>((size_t)3 * nseg * d.NS);
         vfin = carve<T>(6 * d.N);
-        for (int i = 0; i < 2; ++i) ubuf[i] = carve<T>(3 * d.N);
+        for (int i = 0; i < 2; ++i) ubuf[i] = i < two ? carve<T>(3 * d.N) : ubuf[0];
         exact_grad = prm.gradient_mode == LDDMM_GRAD_DISCRETE;
         if (exact_grad) {
             ustore = carve<T>((size_t)3 * (prm.nt + 1) * d.N);
@@ -599,8 +603,12 @@ class Engine : public EngineBase {
         bs1 = (d.n1 - tabs.kcut[1]) & ~1;
         if (bc1 >= bs1) bc1 = bs1 = d.n1;
         if constexpr (sizeof(T) == 4)
-            sl_staged = !force_sl_gather() && raise_smem_limit(k_sl_step_staged<true>, SLBox<true>::SMEM) &&
-                        raise_smem_limit(k_sl_step_staged<false>, SLBox<false>::SMEM);
+            if (!raise_smem_limit(k_sl_step4<true, false>, SLBox<true>::SMEM) ||
+                !raise_smem_limit(k_sl_step4<true, true>, SLBox<true>::SMEM) ||
+                !raise_smem_limit(k_sl_step4<false, false>, SLBox<false>::SMEM) ||
+                !raise_smem_limit(k_sl_step4<false, true>, SLBox<false>::SMEM))
+                return fail(LDDMM_ERR_CUDA);
+        sl_plain = force_sl_gather();
         band_ok = prm.dealias && (fast[0] || gen[0]) && (fast[1] || gen[1]) && !force_generic_fft() &&
                   !force_full_band() && (bnb2 < d.n2h || bc1 < bs1);
         if constexpr (sizeof(T) == 4)
@@ -1114,24 +1122,54 @@ class Engine : public EngineBase {
         return scan_verdict();
     }
 
-    // One semi-Lagrangian map step u0 -> u1 (velocities v0 at t_k, v1 at
-    // t_{k+1}): the shared-memory staged kernel in FP32, the plain gather
-    // kernel in FP64 (or if the staged kernel's shared memory was refused).
-    void sl_step(const GridI& gi, const T* v0, const T* v1, const T* u0, T* u1, T dt_, T ih0, T ih1, T ih2,
-                 int cubic) {
+    // One semi-Lagrangian map step k-1 -> k: velocities vprev at t_{k-1} (FP32: in
+    // packed form from the last step) and v at t_k, both planar.
+    void sl_step(int k, const T* vprev, const T* v) {
+        const GridI gi{d.n0, d.n1, d.n2};
+        const T ih0 = (T)(1.0 / d.h[0]), ih1 = (T)(1.0 / d.h[1]), ih2 = (T)(1.0 / d.h[2]);
+        const bool cubic = prm.interp == LDDMM_INTERP_CUBIC;
+        PScope ps_(this, KC_SL, 12.0 * d.N * sizeof(T));
         if constexpr (sizeof(T) == 4) {
-            if (sl_staged) {
-                const dim3 grid((d.n2 + SLT2 - 1) / SLT2, (d.n1 + SLT1 - 1) / SLT1, (d.n0 + SLT0 - 1) / SLT0);
-                if (cubic)
-                    k_sl_step_staged<true><<<grid, SLT1 * SLT2, SLBox<true>::SMEM, st>>>(gi, v0, v1, u0, u1, dt_, ih0,
-                                                                                          ih1, ih2, d.N);
-                else
-                    k_sl_step_staged<false><<<grid, SLT1 * SLT2, SLBox<false>::SMEM, st>>>(gi, v0, v1, u0, u1, dt_,
-                                                                                            ih0, ih1, ih2, d.N);
-                return;
-            }
+            const bool last = k == prm.nt;
+            const float4 *v0 = sl4[(k - 1) % 2], *u0 = sl4[2 + (k - 1) % 2];
+            float4 *vq = last ? nullptr : sl4[k % 2], *u1q = sl4[2 + k % 2];
+            float* u1p = exact_grad || last ? ubuf_at(k) : nullptr;
+            const dim3 g((d.n2 + SLT2 - 1) / SLT2, (d.n1 + SLT1 - 1) / SLT1, (d.n0 + SLT0 - 1) / SLT0);
+            const size_t sm = cubic ? SLBox<true>::SMEM : SLBox<false>::SMEM;
+            auto go = [&](auto kernel) {
+                kernel<<<g, SLT1 * SLT2, sm, st>>>(gi, v0, v, u0, u1q, vq, u1p, (T)dt(), ih0, ih1, ih2, d.N);
+            };
+            if (sl_plain) cubic ? go(k_sl_step4<true, true>) : go(k_sl_step4<false, true>);
+            else cubic ? go(k_sl_step4<true, false>) : go(k_sl_step4<false, false>);
+        } else {
+            k_sl_step<T><<<pw_grid(d.N), PW_THREADS, 0, st>>>(gi, vprev, v, ubuf_at(k - 1), ubuf_at(k), (T)dt(), ih0,
+                                                             ih1, ih2, cubic, d.N);
         }
-        k_sl_step<T><<<pw_grid(d.N), PW_THREADS, 0, st>>>(gi, v0, v1, u0, u1, dt_, ih0, ih1, ih2, cubic, d.N);
+    }
+    dim3 sl4_grid() const { return dim3((d.n2 + SL4_X - 1) / SL4_X, (d.n1 + SL4_Y - 1) / SL4_Y, d.n0); }
+    // the map at t = 0: u = 0, and v_0 (planar) for the first step
+    void sl_start(const T* v) {
+        if constexpr (sizeof(T) == 4) {
+            if (exact_grad) cudaMemsetAsync(ubuf_at(0), 0, 3 * d.N * sizeof(T), st);
+            cudaMemsetAsync(sl4[2], 0, d.N * sizeof(float4), st);
+            PScope ps_(this, KC_SL, 7.0 * d.N * sizeof(T));
+            k_pack4<<<pw_grid(d.N), PW_THREADS, 0, st>>>(v, sl4[0], d.N);
+        } else {
+            cudaMemsetAsync(ubuf_at(0), 0, 3 * d.N * sizeof(T), st);
+        }
+    }
+    // m1 = I0(x + u1)
+    void warp(const T* I0) {
+        const GridI gi{d.n0, d.n1, d.n2};
+        const T ih0 = (T)(1.0 / d.h[0]), ih1 = (T)(1.0 / d.h[1]), ih2 = (T)(1.0 / d.h[2]);
+        const bool cubic = prm.interp == LDDMM_INTERP_CUBIC;
+        PScope ps_(this, KC_WARP, 5.0 * d.N * sizeof(T));
+        if constexpr (sizeof(T) == 4) {
+            if (cubic) k_warp4<true><<<sl4_grid(), SL4_X * SL4_Y, 0, st>>>(gi, I0, u1(), m1, ih0, ih1, ih2, d.N);
+            else k_warp4<false><<<sl4_grid(), SL4_X * SL4_Y, 0, st>>>(gi, I0, u1(), m1, ih0, ih1, ih2, d.N);
+        } else {
+            k_warp<T><<<pw_grid(d.N), PW_THREADS, 0, st>>>(gi, I0, u1(), m1, ih0, ih1, ih2, cubic, d.N);
+        }
     }
 
     // ------------------------------------------------------------ shooting
@@ -1140,9 +1178,6 @@ class Engine : public EngineBase {
     // k-1 -> k runs too (its velocities are the FP32 copies in vss).
     void shoot_step(int k, const C* cur, C* nxt, bool transport, bool kinetic) {
         const double dt_ = dt();
-        const GridI gi{d.n0, d.n1, d.n2};
-        const T ih0 = (T)(1.0 / d.h[0]), ih1 = (T)(1.0 / d.h[1]), ih2 = (T)(1.0 / d.h[2]);
-        const int cubic = prm.interp == LDDMM_INTERP_CUBIC;
         // Stage fields are evaluated in the compute type: straight into the
         // state store, or into scratch when the store keeps bfloat16 (then
         // k_adstar writes the rounded copy).
@@ -1152,16 +1187,17 @@ class Engine : public EngineBase {
         T* S1 = bf16 ? rs : state(2 * k);
         eval_fields({{cur, 1.0}}, S1);
         if (kinetic) dot_async(S1 + 12 * d.N, S1, 3 * d.N, k, d.cell);
-        if (transport && k >= 1) {
-            PScope ps_(this, KC_SL, 12.0 * d.N * sizeof(T));
-            sl_step(gi, vss[(k - 1) % 2], S1, ubuf_at(k - 1), ubuf_at(k), (T)dt_, ih0, ih1, ih2, cubic);
+        if (transport) {
+            if (k == 0) sl_start(S1);
+            else sl_step(k, vss[(k - 1) % 2], S1);
         }
         {
             PScope ps_(this, KC_ADSTAR, adb);
             k_adstar<T><<<pw_grid(d.N), PW_THREADS, 0, st>>>(StatePtr<T>{S1, d.N}, a, d.N,
                                                             bf16 ? state_bf(2 * k) : nullptr);
         }
-        if (transport) cudaMemcpyAsync(vss[k % 2], S1, 3 * d.N * sizeof(T), cudaMemcpyDeviceToDevice, st);
+        if (transport && sizeof(T) == 8)
+            cudaMemcpyAsync(vss[k % 2], S1, 3 * d.N * sizeof(T), cudaMemcpyDeviceToDevice, st);
         {
             std::vector<FwdOut> outs(3);
             for (int c = 0; c < 3; ++c) {
@@ -1210,13 +1246,8 @@ class Engine : public EngineBase {
     // v0 real -> stores the stage fields, u1 in ubuf[nt%2], kinetic in dres[0..nt]
     void shoot_core(const T* v0, bool kinetic) {
         NvtxRange nr_("lddmm shoot");
-        const double dt_ = dt();
         const int nt = prm.nt;
-        const GridI gi{d.n0, d.n1, d.n2};
-        const T ih0 = (T)(1.0 / d.h[0]), ih1 = (T)(1.0 / d.h[1]), ih2 = (T)(1.0 / d.h[2]);
-        const int cubic = prm.interp == LDDMM_INTERP_CUBIC;
         fwd_vec(v0, v0full);
-        cudaMemsetAsync(ubuf_at(0), 0, 3 * d.N * sizeof(T), st);
         if (band_form) band_copy<true>(v0full, vhat[0]);
         else mask_copy(v0full, v0hat);
         for (int k = 0; k < nt && band_form; ++k) {
@@ -1257,20 +1288,12 @@ class Engine : public EngineBase {
             inverse(srcs, reqs, true);
         }
         if (kinetic) dot_async(vfin + 3 * d.N, vfin, 3 * d.N, nt, d.cell);
-        {
-            PScope ps_(this, KC_SL, 12.0 * d.N * sizeof(T));
-            sl_step(gi, vnat(nt - 1), vfin, ubuf_at(nt - 1), ubuf_at(nt), (T)dt_, ih0, ih1, ih2, cubic);
-        }
+        sl_step(nt, vnat(nt - 1), vfin);
     }
     T* u1() const { return ubuf_at(prm.nt); }
 
     void warp_and_grad(const T* I0) {
-        const GridI gi{d.n0, d.n1, d.n2};
-        {
-            PScope ps_(this, KC_WARP, 5.0 * d.N * sizeof(T));
-            k_warp<T><<<pw_grid(d.N), PW_THREADS, 0, st>>>(gi, I0, u1(), m1, (T)(1.0 / d.h[0]), (T)(1.0 / d.h[1]),
-                                                          (T)(1.0 / d.h[2]), prm.interp == LDDMM_INTERP_CUBIC, d.N);
-        }
+        warp(I0);
         std::vector<FwdOut> outs(1);
         outs[0].out = tmp;
         outs[0].terms.push_back({m1, sym(1.0, 0, -1)});
@@ -1785,8 +1808,6 @@ class Engine : public EngineBase {
     T* vstored(int k) const { return band_sweeps ? vnat(k) : state(2 * k); }
     // One Heun step of the shooting, vhat[0] -> vhat[0], predictor in vhat[1].
     void band_shoot_step(int k, bool transport, bool kinetic) {
-        const GridI gi{d.n0, d.n1, d.n2};
-        const T ih0 = (T)(1.0 / d.h[0]), ih1 = (T)(1.0 / d.h[1]), ih2 = (T)(1.0 / d.h[2]);
         for (int stg = 0; stg < 2; ++stg) {
             C* V = vhat[stg];
             T* S = state(2 * k + stg);
@@ -1798,11 +1819,8 @@ class Engine : public EngineBase {
             plane_inverse(rq, B_IN);
             if (stg == 0 && transport) {
                 nat_inverse(B_IN, 3, vnat(k));
-                if (k >= 1) {
-                    PScope ps_(this, KC_SL, 12.0 * d.N * sizeof(T));
-                    sl_step(gi, vnat(k - 1), vnat(k), ubuf_at(k - 1), ubuf_at(k), (T)dt(), ih0, ih1, ih2,
-                            prm.interp == LDDMM_INTERP_CUBIC);
-                }
+                if (k == 0) sl_start(vnat(0));
+                else sl_step(k, vnat(k - 1), vnat(k));
             }
             stage_run(2, S, 10, 4);
             if (stg == 0 && kinetic) dot_async(S + 3 * d.N, S, 3 * d.N, k, d.cell);
@@ -1939,7 +1957,6 @@ class Engine : public EngineBase {
         const T ih0 = (T)(1.0 / d.h[0]), ih1 = (T)(1.0 / d.h[1]), ih2 = (T)(1.0 / d.h[2]);
         const int cubic = prm.interp == LDDMM_INTERP_CUBIC;
         const int nt = prm.nt;
-        cudaMemsetAsync(vbar, 0, (size_t)3 * (nt + 1) * d.N * sizeof(T), st);
         {
             PScope ps_(this, KC_WARP, 8.0 * d.N * sizeof(T));
             if (cubic)
@@ -1949,25 +1966,47 @@ class Engine : public EngineBase {
                 k_warp_adj<T, false><<<pw_grid(d.N), PW_THREADS, 0, st>>>(gi, I0, u1(), m1, I1, ubar[0], ih0, ih1,
                                                                          ih2, d.N);
         }
-        int cu = 0;
-        for (int k = nt - 1; k >= 0; --k) {
-            cudaMemsetAsync(ubar[1 - cu], 0, 3 * d.N * sizeof(T), st);
-            const T* vk = vstored(k);                            // stage-1 velocity v_k
-            const T* vk1 = k + 1 == nt ? vfin : vstored(k + 1);  // v_{k+1}
-            {
+        if constexpr (sizeof(T) == 4) {
+            // packed copies in the scratch fields: v_k, u_k, dE/du (2), dE/dv (2)
+            float4* const q = (float4*)rs;
+            float4 *const vq = q, *const uq = q + d.N, *const ub = q + 2 * d.N, *const vb = q + 4 * d.N;
+            k_pack4<<<pw_grid(d.N), PW_THREADS, 0, st>>>(ubar[0], ub, d.N);
+            cudaMemsetAsync(vb + (size_t)(nt & 1) * d.N, 0, d.N * sizeof(float4), st);
+            for (int k = nt - 1; k >= 0; --k) {
+                const int cu = (nt - 1 - k) & 1;
+                float4 *const vb0 = vb + (size_t)(k & 1) * d.N, *const vb1 = vb + (size_t)(1 - (k & 1)) * d.N;
+                float4* const ub0 = ub + (size_t)(1 - cu) * d.N;
+                const T* vk1 = k + 1 == nt ? vfin : vstored(k + 1);  // v_{k+1}
                 PScope ps_(this, KC_SL, 24.0 * d.N * sizeof(T));
-                T* vb0 = vbar + (size_t)3 * k * d.N;
-                T* vb1 = vbar + (size_t)3 * (k + 1) * d.N;
-                if (cubic)
-                    k_sl_adj<T, true><<<pw_grid(d.N), PW_THREADS, 0, st>>>(gi, vk, vk1, ubuf_at(k), ubar[cu],
-                                                                          ubar[1 - cu], vb0, vb1, (T)dt(), ih0, ih1,
-                                                                          ih2, d.N);
-                else
-                    k_sl_adj<T, false><<<pw_grid(d.N), PW_THREADS, 0, st>>>(gi, vk, vk1, ubuf_at(k), ubar[cu],
-                                                                           ubar[1 - cu], vb0, vb1, (T)dt(), ih0, ih1,
-                                                                           ih2, d.N);
+                k_pack4<<<pw_grid(d.N), PW_THREADS, 0, st>>>(vstored(k), vq, d.N);
+                k_pack4<<<pw_grid(d.N), PW_THREADS, 0, st>>>(ubuf_at(k), uq, d.N);
+                cudaMemsetAsync(ub0, 0, d.N * sizeof(float4), st);
+                cudaMemsetAsync(vb0, 0, d.N * sizeof(float4), st);
+                auto go = [&](auto kernel) {
+                    kernel<<<sl4_grid(), SL4_X * SL4_Y, 0, st>>>(gi, vq, vk1, uq, ub + (size_t)cu * d.N, ub0, vb0, vb1,
+                                                                (T)dt(), ih0, ih1, ih2, d.N);
+                };
+                cubic ? go(k_sl_adj4<true>) : go(k_sl_adj4<false>);
+                k_unpack4<<<pw_grid(d.N), PW_THREADS, 0, st>>>(vb1, vbar + (size_t)3 * (k + 1) * d.N, d.N);
             }
-            cu = 1 - cu;
+            k_unpack4<<<pw_grid(d.N), PW_THREADS, 0, st>>>(vb, vbar, d.N);
+            return;
+        } else {
+            cudaMemsetAsync(vbar, 0, (size_t)3 * (nt + 1) * d.N * sizeof(T), st);
+            int cu = 0;
+            for (int k = nt - 1; k >= 0; --k) {
+                cudaMemsetAsync(ubar[1 - cu], 0, 3 * d.N * sizeof(T), st);
+                const T* vk = vstored(k);                            // stage-1 velocity v_k
+                const T* vk1 = k + 1 == nt ? vfin : vstored(k + 1);  // v_{k+1}
+                PScope ps_(this, KC_SL, 24.0 * d.N * sizeof(T));
+                auto go = [&](auto kernel) {
+                    kernel<<<pw_grid(d.N), PW_THREADS, 0, st>>>(gi, vk, vk1, ubuf_at(k), ubar[cu], ubar[1 - cu],
+                                                               vbar + (size_t)3 * k * d.N, vbar + (size_t)3 * (k + 1) * d.N,
+                                                               (T)dt(), ih0, ih1, ih2, d.N);
+                };
+                cubic ? go(k_sl_adj<T, true>) : go(k_sl_adj<T, false>);
+                cu = 1 - cu;
+            }
         }
     }
 
@@ -2216,12 +2255,7 @@ class Engine : public EngineBase {
     double energy_at(const T* v, const T* I0, const T* I1) {
         shoot_core(v, false);
         lin_valid = false;
-        const GridI gi{d.n0, d.n1, d.n2};
-        {
-            PScope ps_(this, KC_WARP, 5.0 * d.N * sizeof(T));
-            k_warp<T><<<pw_grid(d.N), PW_THREADS, 0, st>>>(gi, I0, u1(), m1, (T)(1.0 / d.h[0]), (T)(1.0 / d.h[1]),
-                                                          (T)(1.0 / d.h[2]), prm.interp == LDDMM_INTERP_CUBIC, d.N);
-        }
+        warp(I0);
         dot_async(m1, I1, d.N, prm.nt + 2, d.cell, true);
         reg_async(prm.nt + 1);
         if (fetch(0, prm.nt + 3) != LDDMM_OK) return NAN;

@@ -166,9 +166,12 @@ template <class T> __device__ __forceinline__ void cr_weights(T t, T* w) {
     w[3] = (T)0.5 * (t3 - t2);
 }
 
-// Interpolate NC fields (stride N) at voxel (i0,i1,i2) + d (d in voxels).
+// Interpolate NC fields at voxel (i0,i1,i2) + d (d in voxels); component c of
+// grid point o is f[o es + c cs].  The taps of a row along axis 2 are summed
+// first, then the rows (the order that the other kernels below share, so that
+// they agree to the last bit).
 template <class T, int NC>
-__device__ __forceinline__ void interp_at(const T* __restrict__ f, size_t N, GridI g, int i0, int i1, int i2,
+__device__ __forceinline__ void interp_at(const T* __restrict__ f, size_t cs, int es, GridI g, int i0, int i1, int i2,
                                           const T d[3], int cubic, T* res) {
     int base[3];
     T w[3][4];
@@ -192,13 +195,18 @@ __device__ __forceinline__ void interp_at(const T* __restrict__ f, size_t N, Gri
         const size_t o0 = (size_t)wrapi(base[0] + lo + a0, g.n0) * g.n1;
         for (int a1 = 0; a1 < cnt; ++a1) {
             const size_t o1 = (o0 + wrapi(base[1] + lo + a1, g.n1)) * g.n2;
-            const T w01 = w[0][a0] * w[1][a1];
+            T row[NC];
             for (int a2 = 0; a2 < cnt; ++a2) {
-                const size_t o = o1 + wrapi(base[2] + lo + a2, g.n2);
-                const T ww = w01 * w[2][a2];
+                const size_t o = (o1 + wrapi(base[2] + lo + a2, g.n2)) * es;
 #pragma unroll
-                for (int c = 0; c < NC; ++c) res[c] += ww * __ldg(&f[c * N + o]);
+                for (int c = 0; c < NC; ++c) {
+                    const T x = __ldg(&f[c * cs + o]);
+                    row[c] = a2 == 0 ? w[2][0] * x : fma(w[2][a2], x, row[c]);
+                }
             }
+            const T w01 = w[0][a0] * w[1][a1];
+#pragma unroll
+            for (int c = 0; c < NC; ++c) res[c] = fma(w01, row[c], res[c]);
         }
     }
 }
@@ -219,42 +227,91 @@ __global__ void k_sl_step(GridI g, const T* __restrict__ v0, const T* __restrict
             w1[c] = v1[c * N + x];
             d[c] = -dt * w1[c] * ih[c];
         }
-        interp_at<T, 3>(v0, N, g, i0, i1, i2, d, cubic, vt);
+        interp_at<T, 3>(v0, N, 1, g, i0, i1, i2, d, cubic, vt);
         T disp[3];
 #pragma unroll
         for (int c = 0; c < 3; ++c) {
             disp[c] = (T)-0.5 * dt * (w1[c] + vt[c]);
             d[c] = disp[c] * ih[c];
         }
-        interp_at<T, 3>(u0, N, g, i0, i1, i2, d, cubic, ut);
+        interp_at<T, 3>(u0, N, 1, g, i0, i1, i2, d, cubic, ut);
 #pragma unroll
         for (int c = 0; c < 3; ++c) u1[c * N + x] = disp[c] + ut[c];
     }
 }
 
-// ---------------------------------------------------------------- staged map step (FP32)
-// The map step of k_sl_step with its two gathers served from shared memory.
-// A block owns an SLT0 x SLT1 x SLT2 tile of output points.  It stages the
-// sampled field (first v0, then u0) over the tile plus a halo of LO / HI
-// voxels as one float4 (x, y, z, 0) per grid point, so that a tap is one
-// 16-byte shared load instead of three scalar global loads.  A point whose
-// stencil leaves the staged box (more than SL_DMAX voxels of displacement in
-// the step) takes the global gather of interp_at instead, so any velocity is
-// handled; the taps and their summation order are those of interp_at.
-constexpr int SLT0 = 4, SLT1 = 8, SLT2 = 32;  // threads: SLT1 * SLT2 = 256, SLT0 points each
-constexpr int SL_DMAX = 1;                    // staged displacement per step, voxels
+// ---------------------------------------------------------------- map step (FP32)
+// The sampled fields are kept as one float4 (x, y, z, 0) per grid point; a step
+// leaves u1 and v1 in that form for the next one.  A block owns 4 x 8 x 32
+// points and stages the sampled field over them and a halo in shared memory,
+// (x, y) and z apart: 12 bytes a point, and a tap is an 8-byte and a 4-byte
+// load with constant offsets and two packed multiply-adds.  Points whose
+// stencil leaves the box (more than SL_DMAX voxels in the step) gather from
+// global memory in the same order.  Bound by shared memory: 128 taps of 12
+// bytes a point, 87 us at 128^3.  Taps from L1 instead (16-byte loads, no
+// staging) take two cycles where a quarter warp's 128 bytes straddle two
+// lines: 262 us a step.
+constexpr int SLT0 = 4, SLT1 = 8, SLT2 = 32;
+constexpr int SL_DMAX = 1;  // staged displacement per step, voxels
 template <bool CUBIC> struct SLBox {
     static constexpr int TLO = CUBIC ? -1 : 0, CNT = CUBIC ? 4 : 2;  // tap offsets TLO .. TLO + CNT - 1
-    static constexpr int LO = SL_DMAX - TLO;                         // halo below the tile
-    static constexpr int HI = SL_DMAX + TLO + CNT - 1;               // halo above the tile
+    static constexpr int LO = SL_DMAX - TLO, HI = SL_DMAX + TLO + CNT - 1;
     static constexpr int B0 = SLT0 + LO + HI, B1 = SLT1 + LO + HI, B2 = SLT2 + LO + HI;
-    static constexpr int SIZE = B0 * B1 * B2;
-    static constexpr size_t SMEM = (size_t)SIZE * sizeof(float4);
+    // row pitches of whole 128 bytes, so that the lanes of a warp whose stencils
+    // start in different rows still take different banks (without: 49% of the
+    // wavefronts were conflicts)
+    static constexpr int PXY = (B2 + 15) / 16 * 16, PZ = (B2 + 31) / 32 * 32;
+    static constexpr size_t SMEM = (size_t)B0 * B1 * (PXY * 8 + PZ * 4);
 };
-
-// stage the 3 planes of f over the box whose corner is (c0, c1, c2), periodic
+// The stencil of a point with the wrapped offsets of the taps of each axis.
+template <bool CUBIC> struct Sten {
+    static constexpr int CNT = CUBIC ? 4 : 2, LO = CUBIC ? -1 : 0;
+    int o[3][CNT];  // offsets (points) of the taps of each axis
+    float w[3][CNT];
+    // first tap of an axis, wrapped (one period off at most for moderate displacements)
+    static __device__ __forceinline__ int wrap1(int i, int n) {
+        if (i < -n || i >= 2 * n) return wrapi(i, n);
+        return i < 0 ? i + n : (i >= n ? i - n : i);
+    }
+    __device__ __forceinline__ Sten(GridI g, int i0, int i1, int i2, const float d[3]) {
+        const int ii[3] = {i0, i1, i2}, nn[3] = {g.n0, g.n1, g.n2}, st[3] = {g.n1 * g.n2, g.n2, 1};
+#pragma unroll
+        for (int a = 0; a < 3; ++a) {
+            const float fl = floorf(d[a]);
+            const float t = d[a] - fl;
+            int k = wrap1(ii[a] + (int)fl + LO, nn[a]);
+#pragma unroll
+            for (int q = 0; q < CNT; ++q) {
+                o[a][q] = k * st[a];
+                if (++k == nn[a]) k = 0;
+            }
+            if constexpr (CUBIC) {
+                cr_weights(t, w[a]);
+            } else {
+                w[a][0] = 1.f - t;
+                w[a][1] = t;
+            }
+        }
+    }
+};
+__device__ __forceinline__ unsigned long long pk2(float a, float b) {
+    unsigned long long r;
+    asm("mov.b64 %0, {%1, %2};" : "=l"(r) : "f"(a), "f"(b));
+    return r;
+}
+__device__ __forceinline__ unsigned long long fma2u(unsigned long long a, unsigned long long b, unsigned long long c) {
+    unsigned long long r;
+    asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(r) : "l"(a), "l"(b), "l"(c));
+    return r;
+}
+__device__ __forceinline__ unsigned long long mul2u(unsigned long long a, unsigned long long b) {
+    unsigned long long r;
+    asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
+    return r;
+}
+// stage f over the box whose corner is (c0, c1, c2), periodic
 template <bool CUBIC>
-__device__ __forceinline__ void sl_stage(float4* S, const float* __restrict__ f, size_t N, GridI g, int c0, int c1,
+__device__ __forceinline__ void sl_stage(float2* sxy, float* sz, const float4* __restrict__ f, GridI g, int c0, int c1,
                                          int c2) {
     using B = SLBox<CUBIC>;
     // box coordinates lie in [-LO, n + B - LO): within one period of the grid
@@ -262,19 +319,32 @@ __device__ __forceinline__ void sl_stage(float4* S, const float* __restrict__ f,
     // general modulo
     const bool near = g.n0 >= B::B0 && g.n1 >= B::B1 && g.n2 >= B::B2;
     auto wrap = [near](int x, int n) { return near ? (x < 0 ? x + n : (x >= n ? x - n : x)) : wrapi(x, n); };
-    for (int e = threadIdx.x; e < B::SIZE; e += SLT1 * SLT2) {
-        const int b2 = e % B::B2, b1 = (e / B::B2) % B::B1, b0 = e / (B::B2 * B::B1);
-        const size_t o = ((size_t)wrap(c0 + b0, g.n0) * g.n1 + wrap(c1 + b1, g.n1)) * g.n2 + wrap(c2 + b2, g.n2);
-        S[e] = make_float4(__ldg(&f[o]), __ldg(&f[N + o]), __ldg(&f[2 * N + o]), 0.f);
+    // a thread stages the same columns (b1, b2) of every plane b0
+    constexpr int COLS = B::B1 * B::B2, PT = (COLS + SLT1 * SLT2 - 1) / (SLT1 * SLT2);
+    const size_t plane = (size_t)g.n1 * g.n2;
+#pragma unroll
+    for (int q = 0; q < PT; ++q) {
+        const int e = threadIdx.x + q * SLT1 * SLT2;
+        if (e >= COLS) break;
+        const int b1 = e / B::B2, b2 = e - b1 * B::B2;
+        const float4* const p = f + (wrap(c1 + b1, g.n1) * g.n2 + wrap(c2 + b2, g.n2));
+        float4 v[B::B0];
+#pragma unroll
+        for (int b0 = 0; b0 < B::B0; ++b0) v[b0] = __ldg(p + wrap(c0 + b0, g.n0) * plane);
+#pragma unroll
+        for (int b0 = 0; b0 < B::B0; ++b0) {
+            sxy[(b0 * B::B1 + b1) * B::PXY + b2] = make_float2(v[b0].x, v[b0].y);
+            sz[(b0 * B::B1 + b1) * B::PZ + b2] = v[b0].z;
+        }
     }
 }
-
-// the 3 components of the interpolant at (i0,i1,i2) + d: from the staged box
-// when the whole stencil lies in it, else from global memory
+// the interpolant at (i0,i1,i2) + d in interp_at's order: from the staged box
+// when the whole stencil lies in it
 template <bool CUBIC>
-__device__ __forceinline__ void sl_interp(const float4* S, const float* __restrict__ f, size_t N, GridI g, int i0,
-                                          int i1, int i2, int c0, int c1, int c2, const float d[3], float* res) {
+__device__ __forceinline__ void sl_sample(const float2* sxy, const float* sz, const float4* __restrict__ f, GridI g, int i0,
+                                          int i1, int i2, int c0, int c1, int c2, const float d[3], float res[3]) {
     using B = SLBox<CUBIC>;
+    constexpr int CNT = B::CNT;
     int base[3];
     float w[3][4];
     const int ii[3] = {i0, i1, i2};
@@ -291,78 +361,104 @@ __device__ __forceinline__ void sl_interp(const float4* S, const float* __restri
         }
     }
     const int l0 = base[0] + B::TLO - c0, l1 = base[1] + B::TLO - c1, l2 = base[2] + B::TLO - c2;
-    const bool inside = l0 >= 0 && l1 >= 0 && l2 >= 0 && l0 + B::CNT <= B::B0 && l1 + B::CNT <= B::B1 &&
-                        l2 + B::CNT <= B::B2;
+    const bool inside = l0 >= 0 && l1 >= 0 && l2 >= 0 && l0 + CNT <= B::B0 && l1 + CNT <= B::B1 && l2 + CNT <= B::B2;
     if (!inside) {
-        interp_at<float, 3>(f, N, g, i0, i1, i2, d, CUBIC ? 1 : 0, res);
+        interp_at<float, 3>((const float*)f, 1, 4, g, i0, i1, i2, d, CUBIC ? 1 : 0, res);
         return;
     }
-    res[0] = res[1] = res[2] = 0.f;
+    const int r0 = l0 * B::B1 + l1;
+    const unsigned long long* const pxy = (const unsigned long long*)(sxy + r0 * B::PXY + l2);
+    const float* const pz = sz + r0 * B::PZ + l2;
+    unsigned long long xy = 0, w2[CNT];
+    float z = 0.f;
 #pragma unroll
-    for (int a0 = 0; a0 < B::CNT; ++a0) {
+    for (int q = 0; q < CNT; ++q) w2[q] = pk2(w[2][q], w[2][q]);
 #pragma unroll
-        for (int a1 = 0; a1 < B::CNT; ++a1) {
-            const float w01 = w[0][a0] * w[1][a1];
-            const float4* row = S + ((l0 + a0) * B::B1 + (l1 + a1)) * B::B2 + l2;
+    for (int a0 = 0; a0 < CNT; ++a0)
 #pragma unroll
-            for (int a2 = 0; a2 < B::CNT; ++a2) {
-                const float ww = w01 * w[2][a2];
-                const float4 v = row[a2];
-                res[0] += ww * v.x;
-                res[1] += ww * v.y;
-                res[2] += ww * v.z;
+        for (int a1 = 0; a1 < CNT; ++a1) {
+            unsigned long long rxy = 0;
+            float rz = 0.f;
+#pragma unroll
+            for (int a2 = 0; a2 < CNT; ++a2) {
+                const unsigned long long vxy = pxy[(a0 * B::B1 + a1) * B::PXY + a2];
+                const float vz = pz[(a0 * B::B1 + a1) * B::PZ + a2];
+                rxy = a2 == 0 ? mul2u(w2[0], vxy) : fma2u(w2[a2], vxy, rxy);
+                rz = a2 == 0 ? w[2][0] * vz : fmaf(w[2][a2], vz, rz);
             }
+            const float w01 = w[0][a0] * w[1][a1];
+            xy = fma2u(pk2(w01, w01), rxy, xy);
+            z = fmaf(w01, rz, z);
         }
-    }
+    res[0] = __uint_as_float((unsigned)xy);
+    res[1] = __uint_as_float((unsigned)(xy >> 32));
+    res[2] = z;
+}
+// planar field -> float4 per point
+static __global__ void k_pack4(const float* __restrict__ f, float4* __restrict__ out, size_t N) {
+    for (size_t x = blockIdx.x * (size_t)blockDim.x + threadIdx.x; x < N; x += (size_t)gridDim.x * blockDim.x)
+        out[x] = make_float4(f[x], f[N + x], f[2 * N + x], 0.f);
 }
 
-// k_sl_step for FP32 with staged gathers: grid (ceil(n2/SLT2), ceil(n1/SLT1),
-// ceil(n0/SLT0)), SLT1 * SLT2 threads, SLBox<CUBIC>::SMEM dynamic shared bytes
-template <bool CUBIC>
-__global__ void __launch_bounds__(SLT1* SLT2) k_sl_step_staged(GridI g, const float* __restrict__ v0,
-                                                               const float* __restrict__ v1,
-                                                               const float* __restrict__ u0, float* __restrict__ u1,
-                                                               float dt, float ih0, float ih1, float ih2, size_t N) {
+constexpr int SL4_X = 32, SL4_Y = 8;
+// grid (ceil(n2 / SLT2), ceil(n1 / SLT1), ceil(n0 / SLT0)), SLT1 SLT2 threads; v1
+// planar; v1q (nullable): v1 in packed form; u1p: planar copy of u1 (nullable).
+// PLAIN: the loops of interp_at alone (cross-check).
+template <bool CUBIC, bool PLAIN>
+__global__ void __launch_bounds__(SLT1* SLT2, 3) k_sl_step4(GridI g, const float4* __restrict__ v0,
+                                                            const float* __restrict__ v1,
+                                                            const float4* __restrict__ u0, float4* __restrict__ u1,
+                                                            float4* __restrict__ v1q, float* __restrict__ u1p, float dt,
+                                                            float ih0, float ih1, float ih2, size_t N) {
     using B = SLBox<CUBIC>;
     extern __shared__ __align__(16) unsigned char smem_raw[];
-    float4* S = (float4*)smem_raw;
+    float2* const sxy = (float2*)smem_raw;
+    float* const sz = (float*)(sxy + B::B0 * B::B1 * B::PXY);
     const float ih[3] = {ih0, ih1, ih2};
     const int o0 = blockIdx.z * SLT0, o1 = blockIdx.y * SLT1, o2 = blockIdx.x * SLT2;
     const int i1 = o1 + threadIdx.x / SLT2, i2 = o2 + threadIdx.x % SLT2;
     const int c0 = o0 - B::LO, c1 = o1 - B::LO, c2 = o2 - B::LO;  // box corner
     const bool col = i1 < g.n1 && i2 < g.n2;
     float disp[SLT0][3];
-    sl_stage<CUBIC>(S, v0, N, g, c0, c1, c2);
+    if (!PLAIN) sl_stage<CUBIC>(sxy, sz, v0, g, c0, c1, c2);
     __syncthreads();
 #pragma unroll
     for (int p = 0; p < SLT0; ++p) {
         const int i0 = o0 + p;
         if (!col || i0 >= g.n0) continue;
         const size_t x = ((size_t)i0 * g.n1 + i1) * g.n2 + i2;
-        float w1[3], d[3], vt[3];
+        float w1[3], d[3], s[3];
 #pragma unroll
         for (int c = 0; c < 3; ++c) {
-            w1[c] = v1[c * N + x];
+            w1[c] = __ldg(v1 + c * N + x);
             d[c] = -dt * w1[c] * ih[c];
         }
-        sl_interp<CUBIC>(S, v0, N, g, i0, i1, i2, c0, c1, c2, d, vt);
+        if (v1q) v1q[x] = make_float4(w1[0], w1[1], w1[2], 0.f);
+        if constexpr (PLAIN) interp_at<float, 3>((const float*)v0, 1, 4, g, i0, i1, i2, d, CUBIC ? 1 : 0, s);
+        else sl_sample<CUBIC>(sxy, sz, v0, g, i0, i1, i2, c0, c1, c2, d, s);
 #pragma unroll
-        for (int c = 0; c < 3; ++c) disp[p][c] = -0.5f * dt * (w1[c] + vt[c]);
+        for (int c = 0; c < 3; ++c) disp[p][c] = -0.5f * dt * (w1[c] + s[c]);
     }
     __syncthreads();
-    sl_stage<CUBIC>(S, u0, N, g, c0, c1, c2);
+    if (!PLAIN) sl_stage<CUBIC>(sxy, sz, u0, g, c0, c1, c2);
     __syncthreads();
 #pragma unroll
     for (int p = 0; p < SLT0; ++p) {
         const int i0 = o0 + p;
         if (!col || i0 >= g.n0) continue;
         const size_t x = ((size_t)i0 * g.n1 + i1) * g.n2 + i2;
-        float d[3], ut[3];
+        float d[3], s[3];
 #pragma unroll
         for (int c = 0; c < 3; ++c) d[c] = disp[p][c] * ih[c];
-        sl_interp<CUBIC>(S, u0, N, g, i0, i1, i2, c0, c1, c2, d, ut);
+        if constexpr (PLAIN) interp_at<float, 3>((const float*)u0, 1, 4, g, i0, i1, i2, d, CUBIC ? 1 : 0, s);
+        else sl_sample<CUBIC>(sxy, sz, u0, g, i0, i1, i2, c0, c1, c2, d, s);
 #pragma unroll
-        for (int c = 0; c < 3; ++c) u1[c * N + x] = disp[p][c] + ut[c];
+        for (int c = 0; c < 3; ++c) s[c] = disp[p][c] + s[c];
+        u1[x] = make_float4(s[0], s[1], s[2], 0.f);
+        if (u1p) {
+#pragma unroll
+            for (int c = 0; c < 3; ++c) u1p[c * N + x] = s[c];
+        }
     }
 }
 
@@ -378,9 +474,38 @@ __global__ void k_warp(GridI g, const T* __restrict__ img, const T* __restrict__
         T d[3], r[1];
 #pragma unroll
         for (int c = 0; c < 3; ++c) d[c] = u[c * N + x] * ih[c];
-        interp_at<T, 1>(img, N, g, i0, i1, i2, d, cubic, r);
+        interp_at<T, 1>(img, 0, 1, g, i0, i1, i2, d, cubic, r);
         out[x] = r[0];
     }
+}
+// the same in FP32, with the stencil's offsets formed once and its loops
+// unrolled (100 -> 54 us at 128^3); grid (ceil(n2 / 32), ceil(n1 / 8), n0)
+template <bool CUBIC>
+__global__ void __launch_bounds__(SL4_X* SL4_Y) k_warp4(GridI g, const float* __restrict__ img, const float* __restrict__ u,
+                                                        float* __restrict__ out, float ih0, float ih1, float ih2,
+                                                        size_t N) {
+    constexpr int CNT = Sten<CUBIC>::CNT;
+    const int i2 = blockIdx.x * SL4_X + threadIdx.x % SL4_X, i1 = blockIdx.y * SL4_Y + threadIdx.x / SL4_X;
+    const int i0 = blockIdx.z;
+    if (i1 >= g.n1 || i2 >= g.n2) return;
+    const size_t x = ((size_t)i0 * g.n1 + i1) * g.n2 + i2;
+    const float d[3] = {__ldg(u + x) * ih0, __ldg(u + N + x) * ih1, __ldg(u + 2 * N + x) * ih2};
+    const Sten<CUBIC> s(g, i0, i1, i2, d);
+    float r = 0.f;
+#pragma unroll
+    for (int a0 = 0; a0 < CNT; ++a0)
+#pragma unroll
+        for (int a1 = 0; a1 < CNT; ++a1) {
+            const float* const row = img + (s.o[0][a0] + s.o[1][a1]);
+            float q = 0.f;
+#pragma unroll
+            for (int a2 = 0; a2 < CNT; ++a2) {
+                const float v = __ldg(row + s.o[2][a2]);
+                q = a2 == 0 ? s.w[2][0] * v : fmaf(s.w[2][a2], v, q);
+            }
+            r = fmaf(s.w[0][a0] * s.w[1][a1], q, r);
+        }
+    out[x] = r;
 }
 
 // ---------------------------------------------------------------- exact adjoint of the transport
@@ -502,6 +627,7 @@ __global__ void k_warp_adj(GridI g, const T* __restrict__ img, const T* __restri
 // X = x + disp/h, disp = -dt/2 (v1 + v0(p1)), p1 = x - dt v1/h:
 // from ub1 = dE/du_{k+1}, scatter dE/du_k into ub0 and the v0(p1) part of
 // dE/dv_k into vb0 (both atomic), and add the v1 part of dE/dv_{k+1} to vb1.
+// (FP64; FP32 runs k_sl_adj4.)
 template <class T, bool CUBIC>
 __global__ void k_sl_adj(GridI g, const T* __restrict__ v0, const T* __restrict__ v1, const T* __restrict__ u0,
                          const T* __restrict__ ub1, T* ub0, T* vb0, T* __restrict__ vb1, T dt, T ih0, T ih1, T ih2,
@@ -517,7 +643,7 @@ __global__ void k_sl_adj(GridI g, const T* __restrict__ v0, const T* __restrict_
             w1[c] = v1[c * N + x];
             d1[c] = -dt * w1[c] * ih[c];
         }
-        interp_at<T, 3>(v0, N, g, i0, i1, i2, d1, CUBIC ? 1 : 0, vt);
+        interp_at<T, 3>(v0, N, 1, g, i0, i1, i2, d1, CUBIC ? 1 : 0, vt);
         T dX[3];
 #pragma unroll
         for (int c = 0; c < 3; ++c) dX[c] = (T)-0.5 * dt * (w1[c] + vt[c]) * ih[c];
@@ -543,6 +669,130 @@ __global__ void k_sl_adj(GridI g, const T* __restrict__ v0, const T* __restrict_
             vb1[b * N + x] += (T)-0.5 * dt * dispb[b] - dt * ih[b] * p1b;
         }
     }
+}
+
+// float4 per point -> planar field
+static __global__ void k_unpack4(const float4* __restrict__ f, float* __restrict__ out, size_t N) {
+    for (size_t x = blockIdx.x * (size_t)blockDim.x + threadIdx.x; x < N; x += (size_t)gridDim.x * blockDim.x) {
+        const float4 v = f[x];
+        out[x] = v.x;
+        out[N + x] = v.y;
+        out[2 * N + x] = v.z;
+    }
+}
+// weights' derivatives of a stencil
+template <bool CUBIC> struct StenD : Sten<CUBIC> {
+    float dw[3][Sten<CUBIC>::CNT];
+    __device__ __forceinline__ StenD(GridI g, int i0, int i1, int i2, const float d[3]) : Sten<CUBIC>(g, i0, i1, i2, d) {
+#pragma unroll
+        for (int a = 0; a < 3; ++a) {
+            if constexpr (CUBIC) {
+                cr_dweights(d[a] - floorf(d[a]), dw[a]);
+            } else {
+                dw[a][0] = -1.f;
+                dw[a][1] = 1.f;
+            }
+        }
+    }
+};
+// value r[c] and coordinate derivatives G[b][c] of the interpolant of a packed
+// field, the row sums along axis 2 shared between them
+template <bool CUBIC>
+__device__ __forceinline__ void sample4_grad(const float4* __restrict__ f, const StenD<CUBIC>& s, float r[3],
+                                             float (&G)[3][3]) {
+    constexpr int CNT = Sten<CUBIC>::CNT;
+#pragma unroll
+    for (int c = 0; c < 3; ++c) r[c] = G[0][c] = G[1][c] = G[2][c] = 0.f;
+#pragma unroll
+    for (int a0 = 0; a0 < CNT; ++a0)
+#pragma unroll
+        for (int a1 = 0; a1 < CNT; ++a1) {
+            const float4* const row = f + (s.o[0][a0] + s.o[1][a1]);
+            float q[3] = {0.f, 0.f, 0.f}, p[3] = {0.f, 0.f, 0.f};
+#pragma unroll
+            for (int a2 = 0; a2 < CNT; ++a2) {
+                const float4 v = __ldg(row + s.o[2][a2]);
+                const float x[3] = {v.x, v.y, v.z};
+#pragma unroll
+                for (int c = 0; c < 3; ++c) {
+                    q[c] = fmaf(s.w[2][a2], x[c], q[c]);
+                    p[c] = fmaf(s.dw[2][a2], x[c], p[c]);
+                }
+            }
+            const float w01 = s.w[0][a0] * s.w[1][a1], d01 = s.dw[0][a0] * s.w[1][a1], w0d = s.w[0][a0] * s.dw[1][a1];
+#pragma unroll
+            for (int c = 0; c < 3; ++c) {
+                r[c] = fmaf(w01, q[c], r[c]);
+                G[0][c] = fmaf(d01, q[c], G[0][c]);
+                G[1][c] = fmaf(w0d, q[c], G[1][c]);
+                G[2][c] = fmaf(w01, p[c], G[2][c]);
+            }
+        }
+}
+// f[taps] += w x (atomic, 16 bytes a tap)
+template <bool CUBIC>
+__device__ __forceinline__ void scatter4(float4* f, const Sten<CUBIC>& s, const float x[3]) {
+    constexpr int CNT = Sten<CUBIC>::CNT;
+#pragma unroll
+    for (int a0 = 0; a0 < CNT; ++a0)
+#pragma unroll
+        for (int a1 = 0; a1 < CNT; ++a1) {
+            float4* const row = f + (s.o[0][a0] + s.o[1][a1]);
+            const float w01 = s.w[0][a0] * s.w[1][a1];
+#pragma unroll
+            for (int a2 = 0; a2 < CNT; ++a2) {
+                const float w = w01 * s.w[2][a2];
+                atomicAdd(row + s.o[2][a2], make_float4(w * x[0], w * x[1], w * x[2], 0.f));
+            }
+        }
+}
+// k_sl_adj in FP32 on packed fields: a tap is one 16-byte load or atomic instead
+// of three scalar ones, and v0's value and gradient at p1 share their taps.
+// Bound by the atomics: 128 of 16 bytes a point.  Grid as k_warp4.
+template <bool CUBIC>
+__global__ void __launch_bounds__(SL4_X* SL4_Y) k_sl_adj4(GridI g, const float4* __restrict__ v0,
+                                                          const float* __restrict__ v1, const float4* __restrict__ u0,
+                                                          const float4* __restrict__ ub1, float4* ub0, float4* vb0,
+                                                          float4* __restrict__ vb1, float dt, float ih0, float ih1,
+                                                          float ih2, size_t N) {
+    const int i2 = blockIdx.x * SL4_X + threadIdx.x % SL4_X, i1 = blockIdx.y * SL4_Y + threadIdx.x / SL4_X;
+    const int i0 = blockIdx.z;
+    if (i1 >= g.n1 || i2 >= g.n2) return;
+    const size_t x = ((size_t)i0 * g.n1 + i1) * g.n2 + i2;
+    const float ih[3] = {ih0, ih1, ih2};
+    float w1[3], d1[3], vt[3], dX[3], Gv[3][3];
+#pragma unroll
+    for (int c = 0; c < 3; ++c) {
+        w1[c] = __ldg(v1 + c * N + x);
+        d1[c] = -dt * w1[c] * ih[c];
+    }
+    sample4_grad<CUBIC>(v0, StenD<CUBIC>(g, i0, i1, i2, d1), vt, Gv);
+#pragma unroll
+    for (int c = 0; c < 3; ++c) dX[c] = -0.5f * dt * (w1[c] + vt[c]) * ih[c];
+    const float4 ubq = ub1[x];
+    const float ub[3] = {ubq.x, ubq.y, ubq.z};
+    float dispb[3], vtb[3];
+    {
+        const StenD<CUBIC> tX(g, i0, i1, i2, dX);
+        float ut[3], Gu[3][3];
+        sample4_grad<CUBIC>(u0, tX, ut, Gu);
+        scatter4<CUBIC>(ub0, tX, ub);
+#pragma unroll
+        for (int b = 0; b < 3; ++b) {
+            dispb[b] = ub[b] + ih[b] * (Gu[b][0] * ub[0] + Gu[b][1] * ub[1] + Gu[b][2] * ub[2]);
+            vtb[b] = -0.5f * dt * dispb[b];
+        }
+    }
+    scatter4<CUBIC>(vb0, Sten<CUBIC>(g, i0, i1, i2, d1), vtb);
+    float4 o = vb1[x];
+    float add[3];
+#pragma unroll
+    for (int b = 0; b < 3; ++b)
+        add[b] = -0.5f * dt * dispb[b] - dt * ih[b] * (Gv[b][0] * vtb[0] + Gv[b][1] * vtb[1] + Gv[b][2] * vtb[2]);
+    o.x += add[0];
+    o.y += add[1];
+    o.z += add[2];
+    vb1[x] = o;
 }
 
 // ---------------------------------------------------------------- reductions
