@@ -161,6 +161,12 @@ inline void pinned_slots_put(double* p) {
 struct Layout {
     size_t spec_fields, real_fields, bytes;
 };
+// Distance of the components of a spectrum: n0 n1 n2h rounded up to even, so
+// that every component of FP32 pairs starts on a 16-byte boundary (the line
+// kernels of the band form read two entries at once).
+inline size_t spec_stride(const Dims& d) { return (d.NS + 1) & ~(size_t)1; }
+// buffers that an engine carves, each from a 256-byte boundary
+constexpr int MAX_CARVES = POOL + 64;
 inline Layout layout_for(const Dims& d, const lddmm_params* p, size_t tsize) {
     Layout L;
     // pool + vhat(6) + v0hat(3) + v0full(3) + R1(3) + tan(12) + tb(6) + adj(12) + adja(6) + dhat(3) + tmp(3)
@@ -176,19 +182,20 @@ inline Layout layout_for(const Dims& d, const lddmm_params* p, size_t tsize) {
     // exact discrete gradient: every map u_k, every dE/dv_k, two dE/du buffers
     if (p->gradient_mode == LDDMM_GRAD_DISCRETE) L.real_fields += (size_t)6 * (p->nt + 1) + 6;
     if (ckpt) L.spec_fields += (size_t)3 * nseg;  // spectral v at the checkpoints
-    size_t b = L.spec_fields * d.NS * 2 * tsize + L.real_fields * d.N * tsize;
+    size_t b = L.spec_fields * spec_stride(d) * 2 * tsize + L.real_fields * d.N * tsize;
     // stored time states: every stage, or one segment of checkpoint_every steps
     b += (size_t)2 * (ckpt ? cpe : p->nt) * 24 * d.N * (bf16 ? 2 : tsize);
     b += (size_t)(d.n0 + d.n1 + d.n2) * 2 * tsize * 2;  // twiddles
     b += (size_t)(d.n0 + d.n1 + d.n2h) * tsize * 2;      // symbol tables
     b += (RED_BLOCKS * 3 + NSLOT) * sizeof(double);
-    b += 64 * 256;                                       // alignment slack
+    b += (size_t)MAX_CARVES * 256;                       // alignment slack
     L.bytes = b;
     return L;
 }
 
-// LDDMM_GENERIC_FFT=1 selects the generic (runtime-radix) passes for every
-// axis; used to cross-check the register-blocked passes.
+// LDDMM_GENERIC_FFT=1 selects the generic passes of small radices for every axis
+// and the form of the sweeps with all 24 state fields; used to cross-check the
+// register-blocked passes and the band form.
 inline bool force_generic_fft() {
     const char* e = getenv("LDDMM_GENERIC_FFT");
     return e && e[0] == '1';
@@ -435,7 +442,7 @@ class Engine : public EngineBase {
         return b;
     }
 
-    Engine(const Dims& dd, const lddmm_params& p, cudaStream_t s) : d(dd), prm(p), st(s) {}
+    Engine(const Dims& dd, const lddmm_params& p, cudaStream_t s) : d(dd), prm(p), st(s) { d.NS = spec_stride(dd); }
 
     ~Engine() override {
         if (hvg.exec) cudaGraphExecDestroy(hvg.exec);
@@ -614,7 +621,7 @@ class Engine : public EngineBase {
         if constexpr (sizeof(T) == 4)
             fused = bf16 && band_ok && !force_unfused() && FusedPass::has(d.n2) && bnb2 == FusedPass::band_planes(d.n2) &&
                     d.rows % (size_t)FusedPass::tile_rows(d.n2) == 0 && FusedPass::prepare(d.n2);
-        band_form = prm.dealias && !bf16 && band_init();
+        band_form = prm.dealias && !bf16 && !force_generic_fft() && band_init();
         band_sweeps = band_form && !force_unfused() && !force_full_band();
         LD_CK(cudaStreamSynchronize(st));
         return LDDMM_OK;

@@ -1,0 +1,158 @@
+"""The band form of the shooting and the Jacobi sweeps (curl forms of ad* and
+ad on the 2/3-rule band, compiled and run-time line lengths) against the form
+with all 24 state fields and generic passes (LDDMM_GENERIC_FFT=1), and the
+kernels that came with it at the edges of their ranges.
+
+Tolerances: the two forms are equal in exact arithmetic, so in FP64 they
+differ by rounding that the L-weighted terms amplify (1e-10, as against the
+oracle).  In FP32 the 1e-5 of the parity tests holds on axes of up to about 200
+points; beyond, L reaches 5,000 to 30,000 at the edge of the band and the
+24-field form itself is 1e-5 to 1e-4 off in the outputs that carry L, so the
+band form is held to twice that form's own error.
+"""
+import numpy as np
+import pytest
+
+from paper_1807_04638_gb300 import synth
+
+torch = pytest.importorskip("torch")
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module")
+def pkg():
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    import paper_1807_04638_gb300 as p
+    p.lib()
+    return p
+
+
+def rel(a, b):
+    return float(torch.linalg.vector_norm(a.double() - b.double()) / torch.linalg.vector_norm(b.double()))
+
+
+GRIDS = [
+    (16, 18, 16),    # the smallest compiled lengths, a partial tile of rows
+    (27, 25, 45),    # odd row count and odd last axis: run-time radices, single rows
+    (75, 45, 32),    # odd row count, compiled last axis
+    (12, 16, 20),    # axis 0 without compiled line kernels
+    (8, 10, 9),      # two stages of the smallest radices
+    (20, 24, 360),   # last axis without a compiled stage, three stages
+    (18, 400, 24),   # axis 1 beyond the compiled lengths
+    (24, 20, 384),   # the longest compiled stage (4 row pairs a block)
+    (30, 54, 250),   # radices 3 and 5 on every axis
+]
+
+
+def products(pkg, n, prec, nt=2):
+    kmax = max(1, min(3, (min(n) - 1) // 3))
+    I0, vt = synth.blob_pair_inputs(n, 61, kmax=kmax, max_disp_vox=1.5)
+    I0 = synth.spectral_gaussian_smooth(I0, 1.0)
+    I1 = np.roll(I0, 1, axis=2)
+    r = synth.rng_for(62)
+    d, be, bx = (synth.band_limited_field(n, r, 2.0 * kmax, 3) + 0.05 * r.standard_normal((3,) + n) for _ in range(3))
+    dt, cd = (torch.float64, pkg.LDDMM_F64) if prec == "f64" else (torch.float32, pkg.LDDMM_F32)
+    T = lambda a: torch.tensor(np.ascontiguousarray(a), dtype=dt, device="cuda")
+    out = {}
+    for space in (pkg.LDDMM_SPACE_V, pkg.LDDMM_SPACE_L2):
+        prm = pkg.default_params(alpha=0.01, nt=nt, compute_dtype=cd, state_dtype=cd, space=space)
+        with pkg.Handle(n, prm) as h:
+            o = {k: h.new_vec() for k in ("grad", "hv", "eta", "xi", "adj", "vjp")}
+            h.lddmm_gradient(T(0.5 * vt), T(I0), T(I1), o["grad"])
+            h.lddmm_hessvec(T(d), o["hv"])
+            h.lddmm_jacobi_forward(T(d), o["eta"], o["xi"])
+            h.lddmm_jacobi_adjoint(T(be), T(bx), o["adj"])
+            h.lddmm_shoot_vjp(T(I0), o["vjp"])
+            h.lddmm_synchronize()
+            out.update({(k, space): v for k, v in o.items()})
+    return out
+
+
+@pytest.mark.parametrize("n", GRIDS)
+def test_band_form_equals_the_24_field_form(pkg, n, monkeypatch):
+    monkeypatch.setenv("LDDMM_POISON_WORKSPACE", "1")
+    monkeypatch.setenv("LDDMM_GENERIC_FFT", "1")
+    want, want32 = products(pkg, n, "f64"), products(pkg, n, "f32")
+    monkeypatch.delenv("LDDMM_GENERIC_FFT")
+    got, f32 = products(pkg, n, "f64"), products(pkg, n, "f32")
+    for k in want:
+        assert rel(got[k], want[k]) < 1e-10, (k, rel(got[k], want[k]))
+        e, e24 = rel(f32[k], want[k]), rel(want32[k], want[k])
+        assert e < max(1e-5, 2 * e24), (k, e, e24)
+
+
+def spectral_K(x, alpha, s=2):
+    n = x.shape[-3:]
+    k = [torch.fft.fftfreq(m, 1.0 / m, dtype=torch.float64, device=x.device) for m in n[:2]]
+    k.append(torch.fft.rfftfreq(n[2], 1.0 / n[2], dtype=torch.float64, device=x.device))
+    q = k[0][:, None, None] ** 2 + k[1][None, :, None] ** 2 + k[2][None, None, :] ** 2
+    X = torch.fft.rfftn(x.double(), dim=(-3, -2, -1)) / (1.0 + alpha * q) ** s
+    return torch.fft.irfftn(X, s=n, dim=(-3, -2, -1))
+
+
+@pytest.mark.parametrize("prec", ["f64", "f32"])
+@pytest.mark.parametrize("n,comps", [((16, 12, 10), 1), ((16, 12, 10), 30), ((32, 32, 32), 3), ((27, 45, 16), 2),
+                                     ((128, 128, 96), 2)])
+def test_noalloc_takes_components_together(pkg, prec, n, comps):
+    """Groups of components: one, more than a launch's jobs, and a grid whose
+    scratch holds fewer of them than there are; in place too."""
+    dt = torch.float64 if prec == "f64" else torch.float32
+    if prec == "f64" and n[0] == 128:
+        pytest.skip("beyond the fixed scratch in FP64")
+    g = torch.Generator(device="cuda").manual_seed(5)
+    x = torch.randn((comps,) + n, generator=g, dtype=torch.float64, device="cuda").to(dt)
+    want = spectral_K(x, 0.02)
+    out = torch.empty_like(x)
+    pkg.apply_metric_noalloc(x, out, -1, 0.02)
+    tol = 1e-10 if prec == "f64" else 1e-5
+    assert rel(out, want) < tol
+    pkg.apply_metric_noalloc(x, x, -1, 0.02)
+    assert torch.equal(x, out)
+
+
+@pytest.mark.parametrize("prec", ["f64", "f32"])
+@pytest.mark.parametrize("n", [(27, 45, 16), (10, 300, 18), (384, 12, 9), (9, 5, 25)])
+def test_c2c_passes_with_run_time_radices(pkg, prec, n):
+    dt, cd = (torch.float64, pkg.LDDMM_F64) if prec == "f64" else (torch.float32, pkg.LDDMM_F32)
+    g = torch.Generator(device="cuda").manual_seed(6)
+    x = torch.randn((3,) + n, generator=g, dtype=torch.float64, device="cuda").to(dt)
+    out = torch.empty_like(x)
+    with pkg.Handle(n, pkg.default_params(alpha=0.02, nt=1, compute_dtype=cd, state_dtype=cd)) as h:
+        h.lddmm_apply_metric(x, out, -1)
+        h.lddmm_synchronize()
+    assert rel(out, spectral_K(x, 0.02)) < (1e-10 if prec == "f64" else 1e-5)
+
+
+@pytest.mark.parametrize("prec", ["f64", "f32"])
+@pytest.mark.parametrize("off", [0, 1, 3])
+def test_reductions_and_scan_of_unaligned_arrays(pkg, prec, off):
+    """Arrays that start off a 16-byte boundary: the energies equal those of
+    aligned copies to the rounding of a double sum, and a NaN in the first or
+    the last element is found."""
+    n = (9, 10, 5)
+    N = n[0] * n[1] * n[2]
+    dt, cd = (torch.float64, pkg.LDDMM_F64) if prec == "f64" else (torch.float32, pkg.LDDMM_F32)
+    g = torch.Generator(device="cuda").manual_seed(7)
+    prm = pkg.default_params(nt=2, compute_dtype=cd, state_dtype=cd)
+    full = {k: torch.randn(m * N, generator=g, dtype=torch.float64, device="cuda").to(dt)
+            for k, m in (("v", 3), ("a", 1), ("b", 1))}
+    full["v"] *= 0.05
+
+    def shifted(x, shape):
+        y = torch.empty(x.numel() + 4, dtype=dt, device="cuda")
+        y[off:off + x.numel()] = x
+        return y[off:off + x.numel()].view(shape)
+
+    with pkg.Handle(n, prm) as h:
+        grad = h.new_vec()
+        want = h.lddmm_gradient(full["v"].view((3,) + n), full["a"].view(n), full["b"].view(n), grad)
+        got = h.lddmm_gradient(shifted(full["v"], (3,) + n), shifted(full["a"], n), shifted(full["b"], n), grad)
+        assert np.allclose(got, want, rtol=1e-12, atol=0)
+    for at in (0, N - 1):
+        bad = full["b"].clone()
+        bad[at] = float("nan")
+        with pkg.Handle(n, prm) as h:
+            with pytest.raises(pkg.LddmmError) as e:
+                h.lddmm_gradient(full["v"].view((3,) + n), full["a"].view(n), shifted(bad, n), h.new_vec())
+            assert e.value.status == 6
