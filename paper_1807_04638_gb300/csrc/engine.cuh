@@ -12,8 +12,12 @@
 //     through P only; the adjoint state's out-of-band part never reaches its
 //     band, since each operator of the transposed step maps out-of-band
 //     input to out-of-band output);
+//   * the band form of the shooting and the sweeps (stage.cuh, line.cuh,
+//     plane.cuh), taken with P on and states in the compute type: curl forms
+//     of the brackets, 24 line transforms a stage instead of 42;
 //   * EPDiff shooting (Heun) with semi-Lagrangian map transport (Sec. 2.2,
-//     Sec. 3 of the paper), storing every stage's v, Dv, m = Lv, Dm;
+//     Sec. 3 of the paper), storing every stage's v, m = Lv, curl m, div v
+//     (band form) or v, Dv, m, Dm;
 //   * the forward Jacobi (tangent) sweep and its exact transpose, the adjoint
 //     Jacobi sweep (Sec. 3: incremental EPDiff and the reduced (incremental)
 //     adjoint Jacobi equations with the Gauss-Newton drops);
@@ -1592,7 +1596,6 @@ class Engine : public EngineBase {
         bd.b1 = 2 * bd.kc1 + 1;
         bd.nb2 = bd.kc2 + 1;
         bd.fb0 = FastDiv((unsigned)bd.b0);
-        bd.fb1 = FastDiv((unsigned)bd.b1);
         bd.fn1 = FastDiv((unsigned)d.n1);
         bd.b0p = (bd.b0 + 1) & ~1;
         bd.size = (size_t)bd.nb2 * bd.b1 * bd.b0p;

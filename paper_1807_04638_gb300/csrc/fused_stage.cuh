@@ -1,4 +1,7 @@
-// Fused Jacobi stages (FP32 form, band-limited transforms).
+// Fused Jacobi stages of the precision form: FP32 compute with bfloat16
+// states, band-limited transforms.  (States in the compute type take the band
+// form of stage.cuh, with 24 line transforms a stage instead of 42; a
+// bfloat16 state holds the rounded derivatives that these products are of.)
 //
 // One stage of the tangent sweep (Sec. 3, incremental EPDiff and Jacobi
 // field) is: an inverse transform of (eta, xi) into 36 real fields, the
@@ -57,7 +60,7 @@ constexpr int FUSED_BLOCKS = 2;  // resident blocks per SM
 struct FusedArgs {
     const cpx<float>* in[FUSED_NIN];
     cpx<float>* out[FUSED_NOUT];
-    const void* states;     // 24 state fields (float or bfloat16), stride npts
+    const void* states;     // 24 state fields (bfloat16), stride npts
     const float* eta_src;   // adjoint: 3 real fields added to s of group 0, or null
     const float* dk2;       // kappa_2 with the Nyquist entry zeroed (n2/2 + 1)
     const cpx<float>* tw;   // axis-2 twiddles
@@ -105,7 +108,6 @@ template <int N> struct FusedGeom {
     static_assert(!XA || (STG % N == 0 && XT % N == 0), "exchange tiles on line-size boundaries");
 };
 
-__device__ __forceinline__ float ldst(const float* p) { return __ldg(p); }
 __device__ __forceinline__ float ldst(const __nv_bfloat16* p) { return __bfloat162float(__ldg(p)); }
 
 // Stored-state field f of this thread's point m (state layout of pw_kernels.cuh)

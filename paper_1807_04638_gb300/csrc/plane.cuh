@@ -12,9 +12,14 @@
 // they are loaded (a component, a divergence, or a component of a curl, times
 // L, K or 1).  PH = 3 runs both axes on one plane in shared memory, which
 // saves the trip of the half-transformed plane through L2 and its addressing;
-// planes that do not fit (n0 n1 > about 29,000 points in FP32) run the two
-// axes as two launches (PH = 1, then 2; forward 2, then 1) over column and line
-// tiles with the half-transformed band [k2][i1][k0c] between them.
+// FP64 takes it while a plane fits (n0 n1 up to about 14,000 points).  Larger
+// FP64 planes, and all FP32 ones, run the two axes as two launches (PH = 1,
+// then 2; forward 2, then 1) over column and line tiles with the
+// half-transformed band [k2][i1][k0c] between them: a 128^2 FP32 plane leaves
+// an SM one block, and the inverse of a stage at 128^3 took 88 us so against
+// 2 x 38 us in tiles of 16.  Lengths that are compiled in take line.cuh
+// instead: 2 x 24 us.  FP64 is bound by the FP64 rate: its warps wait for that
+// pipe while HBM idles.
 #pragma once
 #include "launch_util.cuh"
 #include "radix.cuh"
@@ -28,7 +33,7 @@ struct Band {
     int b0, p0, b1, p1;
     int b0p;  // row pitch of the spectra: b0 rounded up to even (16-byte rows of FP32 pairs)
     int kc0, kc1, kc2;
-    FastDiv fb0, fb1, fn1;
+    FastDiv fb0, fn1;
     size_t size;  // nb2 b1 b0p
 };
 // index of a band entry on its axis, and back (-1: outside)
@@ -96,6 +101,10 @@ template <class T> struct StepArgs {
     size_t cs;
     T dt;
 };
+// One thread an entry, no shared memory: bound by L2 and HBM (18 to 30
+// band arrays, 2.5 MB each at 128^3).  Apart from the transforms because every
+// output of a vector needs all its components, and a block of line transforms
+// holds lines of one field.
 template <class T, int MODE>
 __global__ void __launch_bounds__(256) k_spec_step(const __grid_constant__ StepArgs<T> a) {
     const Band& bd = a.bd;

@@ -35,8 +35,6 @@
 // (f, f + 1), the even lane transforms f on rows (2i, 2i + 1) and the odd lane
 // f + 1 on the same rows, and one shuffle per point hands each row its own.
 #pragma once
-#include <type_traits>
-
 #include "launch_util.cuh"
 #include "radix.cuh"
 
@@ -71,21 +69,7 @@ inline size_t stage_smem(bool f64, int n2, int lrb) {
     return 16 * (n2 * rb + n2 + 4 * (n2 / 2 + 2) * rb) + 8 * (size_t)n2;
 }
 
-__device__ __forceinline__ float shfl_x1(float v) { return __shfl_xor_sync(0xffffffffu, v, 1); }
 __device__ __forceinline__ double shfl_x1(double v) { return __shfl_xor_sync(0xffffffffu, v, 1); }
-
-// two neighbouring rows of a plane
-__device__ __forceinline__ void ld_pair(const cpx<float>* p, cpx<float>& u, cpx<float>& v) {
-    const float4 q = __ldg((const float4*)p);
-    u = mk(q.x, q.y);
-    v = mk(q.z, q.w);
-}
-__device__ __forceinline__ void ld_pair(const cpx<double>* p, cpx<double>& u, cpx<double>& v) {
-    u = ldg(p);
-    v = ldg(p + 1);
-}
-__device__ __forceinline__ float ldg1(const float* p) { return __ldg(p); }
-__device__ __forceinline__ double ldg1(const double* p) { return __ldg(p); }
 
 template <class T, int P, int KIND>
 __global__ void __launch_bounds__(STAGE_THREADS) k_stage(const __grid_constant__ StageArgs<T> a) {
@@ -105,7 +89,6 @@ __global__ void __launch_bounds__(STAGE_THREADS) k_stage(const __grid_constant__
     const int row = min(row0, rows - 1);
     const bool odd = c & 1;
     const int rA = min((int)blockIdx.x * rb + (c & ~1), (rows - 1) & ~1), dB = rA + 1 < rows ? 1 : 0;
-    const bool vec = (rows & 1) == 0;  // every row pair of a plane is 16-byte aligned (FP32)
     int sel = 0;  // exchange buffer of the next line
     __syncthreads();
 
@@ -113,49 +96,37 @@ __global__ void __launch_bounds__(STAGE_THREADS) k_stage(const __grid_constant__
     auto inv = [&](int f, T(&u)[P], T(&w)[P]) {
         const cpx<T>* const in = a.in[f + (odd ? 1 : 0)] + rA;
         cpx<T>* const buf = buf0 + sel * N * rb + c;
-        auto first = [&](auto pair) {
-            LDDMM_FIRST(pl.a, {
-                const int M = N / R;
-                for (int j = mj; j < M; j += W) {
-                    cpx<T> v[R];
-                    LDDMM_UNROLL
-                    for (int r = 0; r < R; ++r) {
-                        const int k = j + r * M, kn = N - k;
-                        // which half k lies in is known from r but for the middle of an odd radix
-                        const bool hi = 2 * r + 1 == R ? kn < k : 2 * r >= R;
-                        const int kk = hi ? kn : k;
-                        cpx<T> p = mk((T)0, (T)0), q = p;
-                        if (kk < nb2) {
-                            const cpx<T>* s = in + kk * rows;
-                            if constexpr (decltype(pair)::value) {
-                                ld_pair(s, p, q);
-                            } else {
-                                p = ldg(s);
-                                q = ldg(s + dB);
-                            }
-                        }
-                        if ((r == 0 && j == 0) || k == kn) p.y = q.y = (T)0;
-                        if (hi) {
-                            p.y = -p.y;
-                            q.y = -q.y;
-                        }
-                        v[r] = mk(p.x - q.y, p.y + q.x);
+        LDDMM_FIRST(pl.a, {
+            const int M = N / R;
+            for (int j = mj; j < M; j += W) {
+                cpx<T> v[R];
+                LDDMM_UNROLL
+                for (int r = 0; r < R; ++r) {
+                    const int k = j + r * M, kn = N - k;
+                    // which half k lies in is known from r but for the middle of an odd radix
+                    const bool hi = 2 * r + 1 == R ? kn < k : 2 * r >= R;
+                    const int kk = hi ? kn : k;
+                    cpx<T> p = mk((T)0, (T)0), q = p;
+                    if (kk < nb2) {
+                        const cpx<T>* s = in + kk * rows;
+                        p = ldg(s);
+                        q = ldg(s + dB);
                     }
-                    dft<R, 1>(v);
-                    twiddles<R, 1>(v, tws, j);
-                    const int r1 = j / P, j2 = j - r1 * P;
-                    cpx<T>* s = buf + (R * (r1 + pl.b * j2)) * rb;
-                    LDDMM_UNROLL
-                    for (int q = 0; q < R; ++q) s[q * rb] = v[q];
+                    if ((r == 0 && j == 0) || k == kn) p.y = q.y = (T)0;
+                    if (hi) {
+                        p.y = -p.y;
+                        q.y = -q.y;
+                    }
+                    v[r] = mk(p.x - q.y, p.y + q.x);
                 }
-            })
-        };
-        if constexpr (sizeof(T) == 4) {
-            if (vec) first(std::true_type{});
-            else first(std::false_type{});
-        } else {
-            first(std::false_type{});
-        }
+                dft<R, 1>(v);
+                twiddles<R, 1>(v, tws, j);
+                const int r1 = j / P, j2 = j - r1 * P;
+                cpx<T>* s = buf + (R * (r1 + pl.b * j2)) * rb;
+                LDDMM_UNROLL
+                for (int q = 0; q < R; ++q) s[q * rb] = v[q];
+            }
+        })
         __syncthreads();
         if (pl.b > 1) {
             LDDMM_MID(pl.b, {
@@ -256,7 +227,7 @@ __global__ void __launch_bounds__(STAGE_THREADS) k_stage(const __grid_constant__
     };
 
     T* const st0 = a.state ? a.state + (size_t)m * rows + row : nullptr;
-    auto S = [&](int f, int r) { return ldg1(st0 + f * a.npts + (unsigned)(r * W) * (unsigned)rows); };
+    auto S = [&](int f, int r) { return __ldg(st0 + f * a.npts + (unsigned)(r * W) * (unsigned)rows); };
 
     // A: the fields held across the lines of a phase; V (shooting): v and d
     T A[4][P], V[KIND == 2 ? 4 : 1][P], u[P], w[P];
@@ -530,7 +501,12 @@ __global__ void __launch_bounds__(STAGE_THREADS) k_stage(const __grid_constant__
 // line are copied (cp.async) into the other half of a double buffer while the
 // current line is transformed, and the state fields of a line's products are
 // prefetched into L1 when the line begins, so that neither load stands in the
-// chain of a line's barriers.  The last radix is small (3 to 6: the points a
+// chain of a line's barriers.  Bound by shared memory (the LSU is 60% busy) and
+// by the barriers between a line's short steps; DRAM moves 186 MB in the
+// adjoint stage at 128^3.  Adjoint and tangent stage there: 131 us each with
+// one line per thread as in FP64, 107 and 102 packed with run-time radices, 92
+// and 90 compiled; 5 % more with four row pairs a block, 20 % with three
+// blocks an SM (80 registers).  The last radix is small (3 to 6: the points a
 // thread holds), which leaves registers for several blocks per SM.
 __device__ __forceinline__ void put2(float* p, P2 x) { *(float2*)p = make_float2(lo(x), hi(x)); }
 __device__ __forceinline__ P2 get2(const float* p) {
