@@ -12,20 +12,6 @@ template <> struct __align__(16) cpx<double> { double x, y; };
 template <class T> __host__ __device__ __forceinline__ cpx<T> mk(T a, T b) { cpx<T> r; r.x = a; r.y = b; return r; }
 template <class T> __device__ __forceinline__ cpx<T> operator+(cpx<T> a, cpx<T> b) { return mk(a.x + b.x, a.y + b.y); }
 template <class T> __device__ __forceinline__ cpx<T> operator-(cpx<T> a, cpx<T> b) { return mk(a.x - b.x, a.y - b.y); }
-// FP32: both parts in one packed instruction (each part rounded as by the
-// scalar one)
-__device__ __forceinline__ cpx<float> operator+(cpx<float> a, cpx<float> b) {
-    cpx<float> r;
-    asm("{\n .reg .b64 x, y;\n mov.b64 x, {%2, %3};\n mov.b64 y, {%4, %5};\n add.rn.f32x2 x, x, y;\n mov.b64 {%0, %1}, x;\n}"
-        : "=f"(r.x), "=f"(r.y) : "f"(a.x), "f"(a.y), "f"(b.x), "f"(b.y));
-    return r;
-}
-__device__ __forceinline__ cpx<float> operator-(cpx<float> a, cpx<float> b) {
-    cpx<float> r;
-    asm("{\n .reg .b64 x, y;\n mov.b64 x, {%2, %3};\n mov.b64 y, {%4, %5};\n sub.rn.f32x2 x, x, y;\n mov.b64 {%0, %1}, x;\n}"
-        : "=f"(r.x), "=f"(r.y) : "f"(a.x), "f"(a.y), "f"(b.x), "f"(b.y));
-    return r;
-}
 template <class T> __device__ __forceinline__ cpx<T> operator*(cpx<T> a, cpx<T> b) {
     return mk(a.x * b.x - a.y * b.y, a.x * b.y + a.y * b.x);
 }

@@ -348,6 +348,20 @@ class Engine : public EngineBase {
     RPlan gpl[2];
     // band-limited transforms (all three passes register-blocked, dealiasing on)
     bool band_ok = false;
+    // Shooting of a handle with bfloat16 states whose results are L-weighted (the
+    // L2 metric): lengths without a register-blocked plan keep the passes of
+    // radices up to 5 there, over the whole spectrum.  A state that another
+    // summation order moves by an FP32 rounding can round to the other bfloat16
+    // neighbour, and L raises that to 5e-4 of an L2 product at 144 x 192 x 128
+    // (in V, where K takes L out again, 6e-6 at 256 x 300 x 256).
+    bool small_radices = false;
+    struct ShootPasses {
+        Engine* e;
+        explicit ShootPasses(Engine* e_) : e(e_) {
+            e->small_radices = e->bf16 && e->prm.space == LDDMM_SPACE_L2 && (e->gen[0] || e->gen[1]);
+        }
+        ~ShootPasses() { e->small_radices = false; }
+    };
     bool sl_plain = false;  // FP32 map steps by the plain loops (cross-check)
     bool fused = false;      // FP32 Jacobi stages use k_fused_stage
     int bnb2 = 0, bc1 = 0, bs1 = 0;
@@ -681,7 +695,7 @@ class Engine : public EngineBase {
                 const int n = axis == 0 ? d.n0 : (axis == 1 ? d.n1 : d.n2);
                 PScope ps_(this, axis == 0 ? KC_AX0 : (axis == 1 ? KC_AX1 : KC_AX2), pass_bytes(axis, sign, pp_));
                 FastPass<T>::launch(n, axis, sign, pp_, nj, d.rows, d.n0, d.n1, d.n2h, st);
-            } else if (axis < 2 && gen[axis]) {
+            } else if (axis < 2 && gen[axis] && !small_radices) {
                 PScope ps_(this, axis == 0 ? KC_AX0 : KC_AX1, pass_bytes(axis, sign, pp_));
                 GenPass<T>::launch(axis, sign, pp_, nj, gpl[axis], st);
             } else if (axis == 2) {
@@ -795,7 +809,7 @@ class Engine : public EngineBase {
     // The axis-0 and axis-1 passes of inverse(), with the fan-out shared as a
     // tree; the pool's partial spectra hold the results.
     InvHead inverse_head(const std::vector<SpecLin>& srcs, const std::vector<InvReq>& reqs_in, bool band) {
-        const bool bd = band && band_ok;
+        const bool bd = band && band_ok && !small_radices;
         std::vector<InvReq> reqs = reqs_in;
         if (bd)
             for (InvReq& q : reqs) q.sym.mask = 1;
@@ -909,7 +923,7 @@ class Engine : public EngineBase {
         int nin;
     };
     void forward(const std::vector<FwdOut>& outs_in, bool band = false) {
-        const bool bd = band && band_ok;
+        const bool bd = band && band_ok && !small_radices;
         std::vector<FwdOut> outs = outs_in;
         if (bd)
             for (FwdOut& o : outs)
@@ -1242,6 +1256,7 @@ class Engine : public EngineBase {
     void ensure_segment(int j) {
         if (!ckpt || seg_res == j) return;
         seg_res = j;
+        ShootPasses sp_(this);
         const int k0 = j * cpe, k1 = std::min(prm.nt, k0 + cpe);
         if (band_form) {
             band_vec_copy(vhat[0], cps + (size_t)j * 3 * d.NS);
@@ -1258,6 +1273,7 @@ class Engine : public EngineBase {
     void shoot_core(const T* v0, bool kinetic) {
         NvtxRange nr_("lddmm shoot");
         const int nt = prm.nt;
+        ShootPasses sp_(this);
         fwd_vec(v0, v0full);
         if (band_form) band_copy<true>(v0full, vhat[0]);
         else mask_copy(v0full, v0hat);
