@@ -242,7 +242,7 @@ def run_serving(args, dev):
     st = latency_stats(res)
     out = {"requests": len(reqs), "budget_gb": 80, "offered_rate_per_s": 4.0,
            "sizes": [list(r.I0.shape) for r in reqs],
-           "peak_inflight": srv.peak_inflight, "peak_workspace_gb": round(srv.peak_used / 1e9, 2),
+           "peak_inflight": srv.peak_running, "peak_workspace_gb": round(srv.peak_used / 1e9, 2),
            "mse_rel_mean": float(np.mean([r.report["mse_rel"] for r in res if r.report])), **st}
     if args.serve_fp64 > 0:
         # the plain FP64 method and the FP32 form, each serially in FIFO

@@ -153,7 +153,14 @@ class Server:
         self.max_inflight = int(max_inflight)
         self.device = torch.device("cuda", device)
         self.lock = threading.Condition()
-        self.inflight = 0   # slots taken (a finished request's until it is retired)
+        # Two counts.  running: requests admitted and not finished.  inflight:
+        # slots taken, among them those of finished requests that the admission
+        # loop has not taken back yet; it does so when the next request is
+        # admitted, so that peak_inflight says how many slots were needed, not
+        # how many requests ran at the same time (peak_running does).
+        self.running = 0
+        self.peak_running = 0
+        self.inflight = 0
         self.done: List[tuple] = []  # finished, not yet retired: (request, handle, sticky status)
         self.results: Dict[int, Result] = {}
         self.t0 = None
@@ -198,8 +205,7 @@ class Server:
                 res.finished = time.perf_counter() - self.t0
                 with self.lock:
                     self.pool.cancel(hb)
-                    self.done.append((req, None, 0))
-                    self.lock.notify_all()
+                    self._finished(req, None, 0)
                 return
         h, _ = hb
         try:
@@ -222,8 +228,13 @@ class Server:
             if sticky != 0:  # a failed handle is not reused; closed outside the lock
                 h.close()
             with self.lock:
-                self.done.append((req, hb, sticky))
-                self.lock.notify_all()
+                self._finished(req, hb, sticky)
+
+    def _finished(self, req: Request, hb, sticky: int):
+        """Called with the lock held by the worker of a request that ended."""
+        self.running -= 1
+        self.done.append((req, hb, sticky))
+        self.lock.notify_all()
 
     def _retire(self):
         """Called with the lock held: finished requests give up their slots,
@@ -261,20 +272,16 @@ class Server:
                         r = self.results[req.rid]
                         r.status, r.finished = "error: admission deadline exceeded", now
                         continue
-                    # the request takes its slot, then the finished ones give up theirs
-                    self.inflight += 1
-                    self.peak_inflight = max(self.peak_inflight, self.inflight)
+                    slots = self.inflight + 1  # with this request's
                     self._retire()
                     try:
                         hb = self._reserve_handle(req)
                     except Exception as e:
-                        self.inflight -= 1
                         backlog.pop(0)
                         r = self.results[req.rid]
                         r.status, r.finished = f"error: {e}", now
                         continue
                     if hb is None:
-                        self.inflight -= 1
                         if self.inflight == 0:   # can never fit
                             backlog.pop(0)
                             r = self.results[req.rid]
@@ -282,6 +289,10 @@ class Server:
                             continue
                         break
                     backlog.pop(0)
+                    self.inflight += 1
+                    self.peak_inflight = max(self.peak_inflight, slots)
+                    self.running += 1
+                    self.peak_running = max(self.peak_running, self.running)
                     self.results[req.rid].admitted = now
                     t = threading.Thread(target=self._run, args=(req, hb), daemon=True)
                     self.threads.append(t)
