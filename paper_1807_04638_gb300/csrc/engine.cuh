@@ -1937,19 +1937,23 @@ class Engine : public EngineBase {
         for (int c = 0; c < 3; ++c) rq.push_back({adj[0] + c * d.NS, 0, tab, 1.0});
         band_to_real(rq, out);
     }
+    // two real vector fields that share memory (a call in place)
+    bool overlap(const T* a, const T* b) const { return a < b + 3 * d.N && b < a + 3 * d.N; }
     // out = w2 L f + P T^T b (metric L2), or K of it: w2 f + K P T^T b.  F(f)
-    // is read where the sum is taken in the spectrum.
+    // is read where the sum is taken in the spectrum: in L2, and in V when out
+    // shares memory with f, which the sum in real space would read too late.
     void assemble(const T* f, const C* fhat, double w2, int space, T* out) {
         if (!band_sweeps) {
             if (space == LDDMM_SPACE_V) spec_to_real2(fhat, sym(w2, 0, -1), adj_result(), sym(1.0, -1, -1, 1), out);
             else spec_to_real2(fhat, sym(w2, 1, -1), adj_result(), sym(1.0, 0, -1, 1), out);
-        } else if (space == LDDMM_SPACE_V) {
+        } else if (space == LDDMM_SPACE_V && !overlap(f, out)) {
             adj_to_real(out, Kt);
             PScope ps_(this, KC_MISC, 9.0 * d.N * sizeof(T));
             k_axpby<T><<<pw_grid(3 * d.N), PW_THREADS, 0, st>>>((T)w2, f, (T)1, out, 3 * d.N);
         } else {
+            const bool V = space == LDDMM_SPACE_V;
             band_copy<false>(adj[0], adja);
-            spec_to_real2(fhat, sym(w2, 1, -1), adja, sym(1.0, 0, -1, 1), out);
+            spec_to_real2(fhat, sym(w2, V ? 0 : 1, -1), adja, sym(1.0, V ? -1 : 0, -1, 1), out);
         }
     }
 
@@ -2112,8 +2116,8 @@ class Engine : public EngineBase {
 
     void hessvec_core(const T* dv0, T* out, int space) {
         NvtxRange nr_("lddmm hessvec");
-        // the metric L2 adds 2 w L dv0, which needs the whole spectrum of dv0
-        tangent_start(dv0, space == LDDMM_SPACE_L2);
+        // assemble() adds 2 w L dv0 from the whole spectrum of dv0
+        tangent_start(dv0, space == LDDMM_SPACE_L2 || overlap(dv0, out));
         tangent_sweep();
         T* xi = rs;
         tan_to_real(3, xi);
