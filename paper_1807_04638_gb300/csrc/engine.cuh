@@ -177,12 +177,12 @@ inline Layout layout_for(const Dims& d, const lddmm_params* p, size_t tsize) {
     L.spec_fields = POOL + 6 + 3 + 3 + 3 + 12 + 6 + 12 + 6 + 3 + 3;
     // vfin(6) + scratch + m1(1) + gm1(3) + PCG (x r z p q g vt: 21); for the map
     // transport u(6) and the last two stage-1 velocities (6), in FP32 one of
-    // each (6) and both of each with four numbers a point (16)
+    // each (6): both of each, with four numbers a point, lie in tan and adj
     const bool bf16 = p->state_dtype == LDDMM_BF16;
     const int cpe = p->checkpoint_every <= 1 ? p->nt : std::min(p->checkpoint_every, p->nt);
     const bool ckpt = cpe < p->nt;
     const int nseg = (p->nt + cpe - 1) / cpe;
-    L.real_fields = 6 + RSCR + 1 + 3 + 21 + (tsize == 4 ? 22 : 12);
+    L.real_fields = 6 + RSCR + 1 + 3 + 21 + (tsize == 4 ? 6 : 12);
     // exact discrete gradient: every map u_k, every dE/dv_k, two dE/du buffers
     if (p->gradient_mode == LDDMM_GRAD_DISCRETE) L.real_fields += (size_t)6 * (p->nt + 1) + 6;
     if (ckpt) L.spec_fields += (size_t)3 * nseg;  // spectral v at the checkpoints
@@ -522,7 +522,10 @@ class Engine : public EngineBase {
         else states = carve<T>(nstate);
         constexpr int two = sizeof(T) == 4 ? 1 : 2;  // FP32 keeps the last step's fields in sl4
         for (int i = 0; i < 2; ++i) vss[i] = i < two ? carve<T>(3 * d.N) : vss[0];
-        for (int i = 0; i < 4 && sizeof(T) == 4; ++i) sl4[i] = carve<float4>(d.N);
+        // The map steps run in a shooting, outside the sweeps (a segment that a
+        // sweep shoots again takes none), so that their packed fields use the
+        // sweeps' spectra: 16 N bytes in six components of more than 4 N each.
+        for (int i = 0; i < 4 && sizeof(T) == 4; ++i) sl4[i] = (float4*)(i < 2 ? tan_[i] : adj[i - 2]);
         if (ckpt) cps = carve<C>((size_t)3 * nseg * d.NS);
         vfin = carve<T>(6 * d.N);
         for (int i = 0; i < 2; ++i) ubuf[i] = i < two ? carve<T>(3 * d.N) : ubuf[0];
