@@ -259,29 +259,29 @@ struct FusedPass {
     static bool has(int n) { return n == 32 || n == 64 || n == 128 || n == 256; }
     static int tile_rows(int n) { return FAST_THREADS / (n / 8); }
     static int band_planes(int n) { return (n - 1) / 3 + 1; }  // FusedGeom<n>::NB2
-    template <int N, class SS, int KIND> static bool go(const FusedArgs& a, cudaStream_t st, bool set_attr) {
+    template <int N, int KIND> static bool go(const FusedArgs& a, cudaStream_t st, bool set_attr) {
         if (set_attr) {
-            if (!raise_smem_limit(k_fused_stage<SS, N, KIND>, FusedGeom<N>::smem(KIND))) return false;
-            prefer_l1(k_fused_stage<SS, N, KIND>, FusedGeom<N>::smem(KIND), FUSED_BLOCKS);
+            if (!raise_smem_limit(k_fused_stage<N, KIND>, FusedGeom<N>::smem(KIND))) return false;
+            prefer_l1(k_fused_stage<N, KIND>, FusedGeom<N>::smem(KIND), FUSED_BLOCKS);
             return true;
         }
         if (a.nb2 != FusedGeom<N>::NB2) return false;
         const size_t sm = FusedGeom<N>::smem(KIND);
-        k_fused_stage<SS, N, KIND><<<persistent_grid(a.ntiles, FUSED_BLOCKS), FAST_THREADS, sm, st>>>(a);
+        k_fused_stage<N, KIND><<<persistent_grid(a.ntiles, FUSED_BLOCKS), FAST_THREADS, sm, st>>>(a);
         return true;
     }
-    template <class SS, int KIND>
+    template <int KIND>
     static bool launch(int n, const FusedArgs& a, cudaStream_t st, bool set_attr = false) {
         switch (n) {
-            case 32: return go<32, SS, KIND>(a, st, set_attr);
-            case 64: return go<64, SS, KIND>(a, st, set_attr);
-            case 128: return go<128, SS, KIND>(a, st, set_attr);
-            case 256: return go<256, SS, KIND>(a, st, set_attr);
+            case 32: return go<32, KIND>(a, st, set_attr);
+            case 64: return go<64, KIND>(a, st, set_attr);
+            case 128: return go<128, KIND>(a, st, set_attr);
+            case 256: return go<256, KIND>(a, st, set_attr);
             default: return false;
         }
     }
     static bool prepare(int n) {
-        return launch<__nv_bfloat16, 0>(n, FusedArgs{}, 0, true) && launch<__nv_bfloat16, 1>(n, FusedArgs{}, 0, true);
+        return launch<0>(n, FusedArgs{}, 0, true) && launch<1>(n, FusedArgs{}, 0, true);
     }
 };
 
@@ -363,7 +363,7 @@ class Engine : public EngineBase {
         ~ShootPasses() { e->small_radices = false; }
     };
     bool sl_plain = false;  // FP32 map steps by the plain loops (cross-check)
-    bool fused = false;      // FP32 Jacobi stages use k_fused_stage
+    bool fused = false;      // Jacobi stages of bfloat16 states use k_fused_stage
     int bnb2 = 0, bc1 = 0, bs1 = 0;
     // band form (plane.cuh, stage.cuh): dealiasing on, states in the compute type
     bool band_form = false;    // the shooting runs it
@@ -1056,17 +1056,15 @@ class Engine : public EngineBase {
 
     // v, Dv, m = Lv, Dm of a band-limited spectral vector lincomb, into the
     // 24-field layout
-    void eval_fields(std::initializer_list<std::pair<const C*, double>> terms, T* S, bool with_m = true) {
+    void eval_fields(std::initializer_list<std::pair<const C*, double>> terms, T* S) {
         std::vector<SpecLin> srcs;
         std::vector<InvReq> reqs;
         for (int c = 0; c < 3; ++c) srcs.push_back(lin(terms, c));
         for (int c = 0; c < 3; ++c) {
             reqs.push_back({c, sym(1.0, 0, -1), S + c * d.N});
             for (int j = 0; j < 3; ++j) reqs.push_back({c, sym(1.0, 0, j), S + (3 + 3 * c + j) * d.N});
-            if (with_m) {
-                reqs.push_back({c, sym(1.0, 1, -1), S + (12 + c) * d.N});
-                for (int j = 0; j < 3; ++j) reqs.push_back({c, sym(1.0, 1, j), S + (15 + 3 * c + j) * d.N});
-            }
+            reqs.push_back({c, sym(1.0, 1, -1), S + (12 + c) * d.N});
+            for (int j = 0; j < 3; ++j) reqs.push_back({c, sym(1.0, 1, j), S + (15 + 3 * c + j) * d.N});
         }
         inverse(srcs, reqs, true);
     }
@@ -1419,12 +1417,12 @@ class Engine : public EngineBase {
         }
     }
 
-    // ---- fused Jacobi stages (FP32): axis-0/1 passes of the inverse transform,
+    // ---- fused Jacobi stages (bfloat16 states): axis-0/1 passes of the inverse transform,
     // one fused kernel (axis-2 inverse, pointwise products, axis-2 forward),
     // axis-1/0 passes of the forward transform
     void fused_launch(FusedArgs& a, int sidx, int kind) {
         if constexpr (sizeof(T) == 4) {
-            a.states = (const void*)state_bf(sidx);
+            a.states = state_bf(sidx);
             a.dk2 = (const float*)tabs.dk[2];
             a.tw = (const cpx<float>*)ax[2].tw;
             a.rows = (int)d.rows;
@@ -1432,10 +1430,8 @@ class Engine : public EngineBase {
             a.ntiles = (int)(d.rows / (size_t)FusedPass::tile_rows(d.n2));
             a.npts = (unsigned)d.N;
             const double band = (double)bnb2 * d.rows * sizeof(C);
-            const double bytes = 33.0 * band + 24.0 * d.N * state_elem() + (a.eta_src ? 3.0 * d.N * sizeof(T) : 0.0);
-            PScope ps_(this, kind == 0 ? KC_TANF : KC_ADJF, bytes);
-            const bool ok = kind == 0 ? FusedPass::launch<__nv_bfloat16, 0>(d.n2, a, st)
-                                      : FusedPass::launch<__nv_bfloat16, 1>(d.n2, a, st);
+            PScope ps_(this, kind == 0 ? KC_TANF : KC_ADJF, 33.0 * band + 24.0 * d.N * state_elem());
+            const bool ok = kind == 0 ? FusedPass::launch<0>(d.n2, a, st) : FusedPass::launch<1>(d.n2, a, st);
             if (!ok) fail(LDDMM_ERR_DEVICE_CHECK);
         }
     }
@@ -1478,7 +1474,7 @@ class Engine : public EngineBase {
     // outputs per c: groups (s, f) of R'^T without L and under -L into eta_c,
     // of ad_v^T into xi_c, each as (cls 2, cls 0, cls 1) partial spectra
     void adjoint_stage_fused(const std::vector<SpecLin>& srcs, const std::vector<InvReq>& reqs,
-                             const std::vector<FwdOut>& outs, int sidx, const T* eta) {
+                             const std::vector<FwdOut>& outs, int sidx) {
         const InvHead ih = inverse_head(srcs, reqs, true);
         FusedArgs a;
         memset(&a, 0, sizeof(a));
@@ -1497,7 +1493,6 @@ class Engine : public EngineBase {
                     g2.push_back({g < 2 ? c : 3 + c, g == 1 ? 1 : 0, g == 1 ? -1.0 : 1.0, cls, 1, palloc(), 1});
                     a.out[g2.size() - 1] = (cpx<float>*)g2.back().buf;
                 }
-        a.eta_src = (const float*)eta;
         fused_launch(a, sidx, 1);
         forward_tail(outs, g2, true);
     }
@@ -1571,8 +1566,7 @@ class Engine : public EngineBase {
                     }
                 }
                 if (fused) {
-                    adjoint_stage_fused(srcs, reqs, outs, sidx,
-                                        stg == 1 && eta_src ? eta_src + (size_t)3 * k * d.N : nullptr);
+                    adjoint_stage_fused(srcs, reqs, outs, sidx);
                     continue;
                 }
                 inverse(srcs, reqs, true);

@@ -39,8 +39,7 @@
 //   9 groups (s, f_0, f_1, f_2) of the transposed products give 27 outputs,
 //   for c = 0..2 and group g = 0 (R'^T without L), 1 (R'^T under -L),
 //   2 (ad_v^T):  out[9c + 3g] = F2(s) + i kappa_2 F2(f_2),
-//                out[9c + 3g + 1] = F2(f_0), out[9c + 3g + 2] = F2(f_1);
-//   optional real cotangents eta_src (3 fields) are added to s of group 0.
+//                out[9c + 3g + 1] = F2(f_0), out[9c + 3g + 2] = F2(f_1).
 //   Its inverse lines and its (s, f_2) forward lines pack two rows of one
 //   field, as the separate axis-2 pass does (fields of one row can differ
 //   widely in size, and a transform that packed s with f_2 would leave the
@@ -60,8 +59,7 @@ constexpr int FUSED_BLOCKS = 2;  // resident blocks per SM
 struct FusedArgs {
     const cpx<float>* in[FUSED_NIN];
     cpx<float>* out[FUSED_NOUT];
-    const void* states;     // 24 state fields (bfloat16), stride npts
-    const float* eta_src;   // adjoint: 3 real fields added to s of group 0, or null
+    const __nv_bfloat16* states;  // 24 state fields, stride npts
     const float* dk2;       // kappa_2 with the Nyquist entry zeroed (n2/2 + 1)
     const cpx<float>* tw;   // axis-2 twiddles
     int rows, nb2, ntiles;
@@ -111,9 +109,9 @@ template <int N> struct FusedGeom {
 __device__ __forceinline__ float ldst(const __nv_bfloat16* p) { return __bfloat162float(__ldg(p)); }
 
 // Stored-state field f of this thread's point m (state layout of pw_kernels.cuh)
-template <class SS> struct PtState {
-    const SS* p;  // this thread's first point of field 0
-    unsigned n;   // field stride
+struct PtState {
+    const __nv_bfloat16* p;  // this thread's first point of field 0
+    unsigned n;              // field stride
     __device__ __forceinline__ float operator()(int f, int m, int tpl) const { return ldst(p + f * n + tpl * m); }
 };
 // field indices
@@ -151,19 +149,17 @@ __device__ __forceinline__ int line_field(int c, int ty, int q) {
 
 // Bring the state rows of a tile that line (c, type) reads into L1 (one
 // prefetch per 128-byte line), ahead of the loads of its products, so that
-// those loads do not wait on L2; with L2 = true, into L2 only (a line
-// further ahead, so that the L1 prefetch does not wait on DRAM).
-template <class SS, int N, int TL, bool L2 = false>
-__device__ __forceinline__ void prefetch_line_fields(const SS* tile_states, unsigned npts, int c, int ty) {
+// those loads do not wait on L2.
+template <int N, int TL>
+__device__ __forceinline__ void prefetch_line_fields(const __nv_bfloat16* tile_states, unsigned npts, int c, int ty) {
     // the tile's rows of one field are contiguous: PER cache lines
-    constexpr int PER = (int)(TL * N * sizeof(SS) / 128);
-    static_assert(PER * 128 == TL * N * sizeof(SS), "whole cache lines per tile");
+    constexpr int PER = (int)(TL * N * sizeof(__nv_bfloat16) / 128);
+    static_assert(PER * 128 == TL * N * sizeof(__nv_bfloat16), "whole cache lines per tile");
     for (int i = threadIdx.x; i < 6 * PER; i += FAST_THREADS) {
         const int f = line_field(c, ty, i / PER);
         if (f < 0) break;
         const char* p = (const char*)(tile_states + (size_t)f * npts) + (size_t)(i % PER) * 128;
-        if constexpr (L2) asm volatile("prefetch.global.L2 [%0];" ::"l"(p));
-        else asm volatile("prefetch.global.L1 [%0];" ::"l"(p));
+        asm volatile("prefetch.global.L1 [%0];" ::"l"(p));
     }
 }
 
@@ -171,8 +167,8 @@ __device__ __forceinline__ void prefetch_line_fields(const SS* tile_states, unsi
 // acc = (p_0, p_1, p_2, q_0, q_1, q_2):
 //   p_i = m_i div eta + mu_i div v + sum_j (D_i eta_j m_j + D_j m_i eta_j + D_i v_j mu_j + D_j mu_i v_j)
 //   q_i = sum_j (D_j v_i xi_j - D_j xi_i v_j)
-template <int L, int E, int TPL, class SS>
-__device__ __forceinline__ void tan_contrib(float (&acc)[6][E], const cpx<float> (&x)[E], const PtState<SS>& S) {
+template <int L, int E, int TPL>
+__device__ __forceinline__ void tan_contrib(float (&acc)[6][E], const cpx<float> (&x)[E], const PtState& S) {
     constexpr int C = L / 6, TY = L % 6;
 #pragma unroll
     for (int m = 0; m < E; ++m) {
@@ -223,9 +219,8 @@ __device__ __forceinline__ void tan_contrib(float (&acc)[6][E], const cpx<float>
 //   group 1:  s = sum_i D_i v_c y_i + (div v) y_c,  f_j = -v_j y_c
 //   group 2:  s = sum_i D_c v_i yx_i,          f_j = v_j yx_c
 // even types pack (s, f_2), odd types (f_0, f_1).
-template <int F, int E, int TPL, class SS>
-__device__ __forceinline__ void adj_fields(cpx<float> (&x)[E], const float (&acc)[6][E], const PtState<SS>& S,
-                                           const float* eta, unsigned npts) {
+template <int F, int E, int TPL>
+__device__ __forceinline__ void adj_fields(cpx<float> (&x)[E], const float (&acc)[6][E], const PtState& S) {
     constexpr int C = F / 6, TY = F % 6;
     const float(&y)[6][E] = acc;  // y_i = acc[i], yx_i = acc[3 + i]
 #pragma unroll
@@ -240,7 +235,6 @@ __device__ __forceinline__ void adj_fields(cpx<float> (&x)[E], const float (&acc
                 a = 0.f;
 #pragma unroll
                 for (int i = 0; i < 3; ++i) a -= S(fDm(i, C), m, TPL) * y[i][m];
-                if (eta) a += __ldg(eta + C * npts + TPL * m);
                 b = mC * y[2][m] + (C == 2 ? my : 0.f);
             } else {
                 a = mC * y[0][m] + (C == 0 ? my : 0.f);
@@ -329,7 +323,7 @@ template <int KIND> __device__ __forceinline__ void fused_line_inputs(int l, int
     }
 }
 
-template <class SS, int N, int KIND>
+template <int N, int KIND>
 __global__ void __launch_bounds__(FAST_THREADS, FUSED_BLOCKS) k_fused_stage(const __grid_constant__ FusedArgs a) {
     using G = FusedGeom<N>;
     constexpr int E = G::E, TPL = G::TPL, TL = G::TL, NH = G::NH, SP = G::SP, PH = G::PH, RP = G::RP, FS = G::FS;
@@ -390,12 +384,12 @@ __global__ void __launch_bounds__(FAST_THREADS, FUSED_BLOCKS) k_fused_stage(cons
         issue(tl2, l2, d);
     }
     int sb = 0;
-    const SS* const states = (const SS*)a.states;
+    const __nv_bfloat16* const states = a.states;
     cpx<float> x[E];
     for (; tile < ntiles; tile += gridDim.x) {
         const int r0 = tile * TL;
-        const SS* const tile_states = states + (size_t)r0 * N;
-        const PtState<SS> S{states + (size_t)(r0 + c) * N + t, a.npts};
+        const __nv_bfloat16* const tile_states = states + (size_t)r0 * N;
+        const PtState S{states + (size_t)(r0 + c) * N + t, a.npts};
         // tangent: p, q accumulators; adjoint: y, yx
         float acc[6][E];
 #pragma unroll
@@ -416,7 +410,7 @@ __global__ void __launch_bounds__(FAST_THREADS, FUSED_BLOCKS) k_fused_stage(cons
             }
             const cpx<float>* const stg = stage0 + sb * STG;
             if constexpr (KIND == 0) {
-                prefetch_line_fields<SS, N, TL>(tile_states, a.npts, l / 6, l % 6);
+                prefetch_line_fields<N, TL>(tile_states, a.npts, l / 6, l % 6);
                 // two fields of this line group's row: (in[i0], D2 in[i0]) or (in[i0], in[i1])
                 int i0, i1;
                 fused_line_inputs<KIND>(l, i0, i1);
@@ -447,7 +441,7 @@ __global__ void __launch_bounds__(FAST_THREADS, FUSED_BLOCKS) k_fused_stage(cons
                     }
                 }
             } else {
-                if (l == NLI - 1) prefetch_line_fields<SS, N, TL>(tile_states, a.npts, 0, 0);
+                if (l == NLI - 1) prefetch_line_fields<N, TL>(tile_states, a.npts, 0, 0);
                 // one field (input q of the line) on a pair of rows
                 // the row pair's two entries are adjacent: one 16-byte load
                 const float4* SA = (const float4*)(stg + q * nb2 * SP + 2 * rp);
@@ -510,17 +504,16 @@ __global__ void __launch_bounds__(FAST_THREADS, FUSED_BLOCKS) k_fused_stage(cons
                     else x[m] = mk(acc[4][m], acc[5][m]);
                 }
             } else {
-                const float* eta = a.eta_src ? a.eta_src + (size_t)(r0 + c) * N + t : nullptr;
                 switch (f) {
 #define LDDMM_AF(F) \
-    case F: adj_fields<F, E, TPL>(x, acc, S, eta, a.npts); break;
+    case F: adj_fields<F, E, TPL>(x, acc, S); break;
                     LDDMM_AF(0) LDDMM_AF(1) LDDMM_AF(2) LDDMM_AF(3) LDDMM_AF(4) LDDMM_AF(5)
                     LDDMM_AF(6) LDDMM_AF(7) LDDMM_AF(8) LDDMM_AF(9) LDDMM_AF(10) LDDMM_AF(11)
                     LDDMM_AF(12) LDDMM_AF(13) LDDMM_AF(14) LDDMM_AF(15) LDDMM_AF(16) LDDMM_AF(17)
 #undef LDDMM_AF
                     default: break;
                 }
-                if (f + 1 < NLO) prefetch_line_fields<SS, N, TL>(tile_states, a.npts, (f + 1) / 6, (f + 1) % 6);
+                if (f + 1 < NLO) prefetch_line_fields<N, TL>(tile_states, a.npts, (f + 1) / 6, (f + 1) % 6);
                 if (f % 2 == 0) {
                     // (s, f_2): the two fields go to the line groups that
                     // transform them on row pairs (two rows of one field share
