@@ -7,9 +7,11 @@ GPU.  Run ``python -m paper_1807_04638_gb300.build`` or call ``build()``.
 from __future__ import annotations
 
 import os
+import re
 import shutil
 import subprocess
 import sys
+from concurrent.futures import ThreadPoolExecutor
 
 HERE = os.path.dirname(os.path.abspath(__file__))
 ROOT = os.path.dirname(HERE)
@@ -19,6 +21,14 @@ OUT_DIR = os.path.join(HERE, "lib")
 BUILD_DIR = os.path.join(HERE, "_build")
 LIB = os.path.join(OUT_DIR, "liblddmm.so")
 
+
+def stage_lengths():
+    """The compiled line lengths, longest first: LDDMM_STAGE_LENGTHS of stage.cuh."""
+    with open(os.path.join(CSRC, "stage.cuh")) as f:
+        table = re.search(r"#define LDDMM_STAGE_LENGTHS\(X\)((?:.*\\\n)*.*\n)", f.read()).group(1)
+    return sorted((int(n) for n in re.findall(r"X\((\d+),", table)), reverse=True)
+
+
 # (source, object, defines): the passes are compiled once per number type, the
 # stage kernels once per number type and last radix, the kernels of a compiled
 # length once per length
@@ -27,8 +37,7 @@ SOURCES = [(f"{s}.cu", f"{s}_{t}.o", (f"-DLDDMM_T={t}",))
 SOURCES += [(f"{s}.cu", f"{s}.o", ()) for s in ("engine_f32", "engine_f64", "noalloc", "capi", "probe")]
 SOURCES += [("stage_radix.cu", f"stage_{t}_{p}.o", (f"-DLDDMM_STAGE_T={t}", f"-DLDDMM_STAGE_P={p}"))
             for t, ps in (("float", (6, 5, 4, 3)), ("double", (10, 9, 8, 6, 5, 4))) for p in ps]
-STAGE_LENGTHS = [384, 320, 300, 288, 270, 256, 250, 243, 240, 225, 216, 200, 192, 180, 162, 160, 150, 144, 135, 128, 125, 120, 108, 100, 96, 90, 81, 80, 75, 72, 64, 60, 54, 50, 48, 45, 40, 36, 32, 30, 27, 25, 24, 20, 18, 16]
-SOURCES += [("stage_length.cu", f"stage_n{n}.o", (f"-DLDDMM_STAGE_N={n}",)) for n in STAGE_LENGTHS]
+SOURCES += [("stage_length.cu", f"stage_n{n}.o", (f"-DLDDMM_STAGE_N={n}",)) for n in stage_lengths()]
 ARCH = ["-gencode", "arch=compute_103a,code=sm_103a"]
 
 
@@ -49,22 +58,24 @@ def build(verbose: bool = False, extra_flags=()) -> str:
     nvcc = nvcc_path()
     os.makedirs(OUT_DIR, exist_ok=True)
     os.makedirs(BUILD_DIR, exist_ok=True)
-    procs = []
     objs = []
+    cmds = []
     for src, name, defines in SOURCES:
         obj = os.path.join(BUILD_DIR, name)
         objs.append(obj)
         cmd = [nvcc, *_flags(extra_flags), *defines, "-c", os.path.join(CSRC, src), "-o", obj]
         if verbose:
             print(" ".join(cmd), flush=True)
-        procs.append((name, subprocess.Popen(cmd, stdout=subprocess.PIPE, stderr=subprocess.STDOUT)))
+        cmds.append(cmd)
+    # one compiler per core at a time
     failed = []
-    for src, p in procs:
-        out, _ = p.communicate()
-        if p.returncode != 0 or verbose:
-            sys.stderr.write(out.decode(errors="replace"))
-        if p.returncode != 0:
-            failed.append(src)
+    run = lambda cmd: subprocess.run(cmd, stdout=subprocess.PIPE, stderr=subprocess.STDOUT)
+    with ThreadPoolExecutor(os.cpu_count() or 1) as ex:
+        for (src, name, _), p in zip(SOURCES, ex.map(run, cmds)):
+            if p.returncode != 0 or verbose:
+                sys.stderr.write(p.stdout.decode(errors="replace"))
+            if p.returncode != 0:
+                failed.append(name)
     if failed:
         raise RuntimeError(f"nvcc failed for {failed}")
     tmp = LIB + ".tmp"
