@@ -147,22 +147,32 @@ def workload_inputs(n=N128, seed=1):
     return P, v0, e0, e1, d
 
 
-# DRAM traffic per launch of the stage kernels, from an ncu capture
-# (profiles/band_form_128cubed_f32_ncu.md; one launch is one stage over the
-# whole grid, the same at every nt), valid only for the kernel sources it was
-# measured on: reported as null once the sources change.
-TRAFFIC = {"digest": "6284b35898e063f8", "adjoint_stage_fused": 186.4e6, "tangent_stage_fused": 197.0e6}
+# DRAM traffic per launch of the dominant kernel classes, read and written, from an
+# ncu capture of one product (profiles/band_form_128cubed_f32_ncu.md; the caches as
+# the product leaves them; the line kernels averaged over the launches of a product
+# at nt = 10).  Valid only for the kernel code it was measured on: reported as null
+# once that changes.
+TRAFFIC = {"digest": "7754d3ce8ca2c7a9", "adjoint_stage_fused": 229.1e6, "tangent_stage_fused": 240.6e6,
+           "fft_plane_inverse": 56.0e6, "fft_plane_forward": 55.2e6}
 
 
-def kernel_digest():
-    """Digest of the stage-kernel sources (the dominant kernel classes): a
-    stored DRAM-traffic figure holds only for this digest."""
+def kernel_digest(csrc=os.path.join(ROOT, "paper_1807_04638_gb300", "csrc")):
+    """Digest of the code of the stage and line kernels of a compiled length and
+    of everything they include, without comments and white space: a stored
+    DRAM-traffic figure holds only for this digest."""
     import hashlib
+    import re
     h = hashlib.sha1()
-    csrc = os.path.join(ROOT, "paper_1807_04638_gb300", "csrc")
-    for f in ("common.cuh", "radix.cuh", "stage.cuh"):
-        with open(os.path.join(csrc, f), "rb") as fh:
-            h.update(fh.read())
+    todo, seen = ["stage_length.cu"], set()
+    while todo:
+        f = todo.pop(0)
+        if f in seen or not os.path.exists(os.path.join(csrc, f)):
+            continue
+        seen.add(f)
+        with open(os.path.join(csrc, f), encoding="utf-8") as fh:
+            src = re.sub(r"/\*.*?\*/|//[^\n]*", "", fh.read(), flags=re.S)
+        todo += re.findall(r'#include "([^"]+)"', src)
+        h.update((f + "".join(src.split())).encode())
     return h.hexdigest()[:16]
 
 
@@ -535,7 +545,7 @@ def profile_run(h, delta, hv, value, world):
     roofline = {"bound": "hbm", "kernel": dom, "achieved": round(achieved, 1) if achieved else None,
                 "peak": peak, "peak_kind": peak_kind + " hbm_gbs (STREAM-style copy)", "unit": "GB/s",
                 "frac": round(achieved / peak, 4) if achieved else None,
-                "traffic": TRAFFIC.get(dom) if TRAFFIC["digest"] == kernel_digest() else None,
+                "traffic": TRAFFIC.get(dom) if h.n == N128 and TRAFFIC["digest"] == kernel_digest() else None,
                 "kernel_digest": kernel_digest(),
                 "algorithmic_bytes_per_launch": dbytes / dn if dn else None,
                 "path_frac_compulsory_5GB_per_hv": round(value / world * 5.0e9 / (peak * 1e9), 4)}
