@@ -11,6 +11,7 @@
 #include <cuda_bf16.h>
 
 #include "common.cuh"
+#include "radix.cuh"
 
 namespace lddmm {
 
@@ -294,21 +295,6 @@ template <bool CUBIC> struct Sten {
         }
     }
 };
-__device__ __forceinline__ unsigned long long pk2(float a, float b) {
-    unsigned long long r;
-    asm("mov.b64 %0, {%1, %2};" : "=l"(r) : "f"(a), "f"(b));
-    return r;
-}
-__device__ __forceinline__ unsigned long long fma2u(unsigned long long a, unsigned long long b, unsigned long long c) {
-    unsigned long long r;
-    asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(r) : "l"(a), "l"(b), "l"(c));
-    return r;
-}
-__device__ __forceinline__ unsigned long long mul2u(unsigned long long a, unsigned long long b) {
-    unsigned long long r;
-    asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
-    return r;
-}
 // stage f over the box whose corner is (c0, c1, c2), periodic
 template <bool CUBIC>
 __device__ __forceinline__ void sl_stage(float2* sxy, float* sz, const float4* __restrict__ f, GridI g, int c0, int c1,
@@ -367,31 +353,31 @@ __device__ __forceinline__ void sl_sample(const float2* sxy, const float* sz, co
         return;
     }
     const int r0 = l0 * B::B1 + l1;
-    const unsigned long long* const pxy = (const unsigned long long*)(sxy + r0 * B::PXY + l2);
+    const P2* const pxy = (const P2*)(sxy + r0 * B::PXY + l2);
     const float* const pz = sz + r0 * B::PZ + l2;
-    unsigned long long xy = 0, w2[CNT];
+    P2 xy = p2(0.f, 0.f), w2[CNT];
     float z = 0.f;
 #pragma unroll
-    for (int q = 0; q < CNT; ++q) w2[q] = pk2(w[2][q], w[2][q]);
+    for (int q = 0; q < CNT; ++q) w2[q] = p2(w[2][q], w[2][q]);
 #pragma unroll
     for (int a0 = 0; a0 < CNT; ++a0)
 #pragma unroll
         for (int a1 = 0; a1 < CNT; ++a1) {
-            unsigned long long rxy = 0;
+            P2 rxy = p2(0.f, 0.f);
             float rz = 0.f;
 #pragma unroll
             for (int a2 = 0; a2 < CNT; ++a2) {
-                const unsigned long long vxy = pxy[(a0 * B::B1 + a1) * B::PXY + a2];
+                const P2 vxy = pxy[(a0 * B::B1 + a1) * B::PXY + a2];
                 const float vz = pz[(a0 * B::B1 + a1) * B::PZ + a2];
-                rxy = a2 == 0 ? mul2u(w2[0], vxy) : fma2u(w2[a2], vxy, rxy);
+                rxy = a2 == 0 ? w2[0] * vxy : fma2(w2[a2], vxy, rxy);
                 rz = a2 == 0 ? w[2][0] * vz : fmaf(w[2][a2], vz, rz);
             }
             const float w01 = w[0][a0] * w[1][a1];
-            xy = fma2u(pk2(w01, w01), rxy, xy);
+            xy = fma2(p2(w01, w01), rxy, xy);
             z = fmaf(w01, rz, z);
         }
-    res[0] = __uint_as_float((unsigned)xy);
-    res[1] = __uint_as_float((unsigned)(xy >> 32));
+    res[0] = lo(xy);
+    res[1] = hi(xy);
     res[2] = z;
 }
 // planar field -> float4 per point
