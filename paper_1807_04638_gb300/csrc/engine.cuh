@@ -2064,13 +2064,13 @@ class Engine : public EngineBase {
         assemble(v0, v0full, w2, space, grad);
         lin_valid = true;
     }
-    // ---- the Hessian-vector product as a CUDA graph.  Its ~220 launches
-    // depend only on the handle and on (dv0, out, space): they are recorded
-    // once (stream capture) and replayed, which removes the gaps between
-    // back-to-back launches.  Not with the profiler on (it times each
-    // launch), with checkpointed states (the re-shooting depends on which
-    // segment is resident), or when the stream cannot be captured (the
-    // legacy default stream): then the kernels are launched one by one.
+    // ---- the Hessian-vector product as a CUDA graph.  Its launches (255 at
+    // nt = 10 in the band form) depend only on the handle and on (dv0, out,
+    // space): they are recorded once (stream capture) and replayed, which removes
+    // the gaps between back-to-back launches.  Not with the profiler on (it times
+    // each launch), with checkpointed states (the re-shooting depends on which
+    // segment is resident), or when the stream cannot be captured (the legacy
+    // default stream): then the kernels are launched one by one.
     struct HvGraph {
         const void* in = nullptr;
         void* out = nullptr;

@@ -62,8 +62,10 @@ inline int persistent_grid(int items, int per_sm = 3) {
 // or reads, and dependents_may_launch() when it is about to write its last
 // results: at that point the launch latency and the prologue are hidden and
 // the dependents take no room from its own blocks.  Hessian-vector product at
-// 64^3: 1.52 ms without, 1.42 ms so, 1.64 ms with the call at the kernel's
-// start; at 128^3 7.11, 6.97 and 6.91 ms.
+// 64^3: 1.52 ms without, 1.42 ms so, 1.64 ms with the call at every kernel's
+// start; at 128^3 7.11, 6.97 and 6.91 ms.  k_spec_step alone calls it first: it
+// has no prologue worth the name and its blocks no shared memory, and the place
+// makes no difference there (1,417 us at 64^3 and 6,973 us at 128^3 either way).
 template <class A>
 inline void launch_dependent(void (*kernel)(A), dim3 grid, unsigned threads, size_t smem, cudaStream_t st, const A& a) {
     cudaLaunchConfig_t cfg = {};

@@ -16,9 +16,11 @@
 // kernels: a warp's 8-byte accesses cover four neighbouring k0c of eight lines,
 // whole 32-byte sectors.
 //
-// Bound by HBM and L2: about 5 TB/s of algorithmic bytes a launch.  At 128^3 a
-// launch of a stage's inverse takes 24 us on average (38 us with run-time
-// radices, 35 us with the band's limits taken from the arguments); radices of
+// Bound by the latency of their loads (long_scoreboard; 13 warps an SM, as many
+// as the registers leave room for): 4.4 TB/s of algorithmic bytes a launch
+// inverse, 4.1 forward.  At 128^3 a launch takes 23 us on average inverse and 22
+// forward (an inverse one 38 us with run-time radices, 35 us with the band's
+// limits taken from the arguments); radices of
 // at most 10 or 8 make the whole product 16 % slower (more exchanges), 10 or 12
 // blocks of 64 threads an SM the launch 12 to 14 % (registers).
 #pragma once

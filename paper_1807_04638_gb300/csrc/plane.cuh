@@ -18,7 +18,7 @@
 // half-transformed band [k2][i1][k0c] between them: a 128^2 FP32 plane leaves
 // an SM one block, and the inverse of a stage at 128^3 took 88 us so against
 // 2 x 38 us in tiles of 16.  Lengths that are compiled in take line.cuh
-// instead: 2 x 24 us.  FP64 is bound by the FP64 rate: its warps wait for that
+// instead: 2 x 23 us.  FP64 is bound by the FP64 rate: its warps wait for that
 // pipe while HBM idles.
 #pragma once
 #include "launch_util.cuh"
@@ -108,7 +108,7 @@ template <class T> struct StepArgs {
 template <class T, int MODE>
 __global__ void __launch_bounds__(256) k_spec_step(const __grid_constant__ StepArgs<T> a) {
     const Band& bd = a.bd;
-    dependents_may_launch();
+    dependents_may_launch();  // see launch_util.cuh
     after_previous();
     const int i = blockIdx.x * 256 + threadIdx.x;
     if (i >= (int)bd.size) return;

@@ -4,7 +4,8 @@
 // map step and of the warp (discrete gradient), Jacobian determinants and
 // double-precision reductions.
 //
-// A time state holds 24 real fields, each N = n0*n1*n2 values:
+// A time state holds 24 real fields, each N = n0*n1*n2 values (the band form's
+// ten are in stage.cuh):
 //   [0..2]   v_c          [3 + 3c + j]  D_j v_c
 //   [12..14] m_c = (L v)_c [15 + 3c + j] D_j m_c
 #pragma once

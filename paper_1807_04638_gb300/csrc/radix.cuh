@@ -234,9 +234,9 @@ constexpr int RP_FIRST[] = {2, 3, 4, 5, 6, 8, 9, 10, 12, 15, 16};  // radices of
 constexpr int RP_MID[] = {2, 3, 4, 5, 6, 8, 9, 10};                // of the middle stage
 
 // The plan with the fewest stages and, among those, the smallest largest
-// radix (registers); n = 0 when there is none (n < 8, and lengths with a
-// factor that no radix covers).  few: last radix 3 to 6, the others at most 10
-// (the FP32 stage kernels).
+// radix (registers); n = 0 when there is none.  Every length up to 512 with
+// factors 2, 3 and 5 has one but those below 8, and 9.  few: last radix 3 to 6,
+// the others at most 10 (the FP32 stage kernels); none for 375 and 512 either.
 inline RPlan radix_plan3(int n, bool few = false) {
     RPlan best;
     int score = 1 << 30;

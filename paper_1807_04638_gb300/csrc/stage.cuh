@@ -56,8 +56,8 @@ constexpr int STAGE2_THREADS = 512; // at most (FP32; 128 registers)
 // row pairs of a block (FP32): 8 (128-byte segments of a plane) while that is at
 // most 256 threads, else 4, so that two blocks and more share an SM
 __host__ __device__ constexpr int stage_rb(int n, int p) { return n / p * 8 <= 256 ? 8 : 4; }
-// blocks per SM that leave a thread 128 registers (fewer registers spill: 80
-// made the 128^3 adjoint stage 15% slower)
+// blocks per SM that leave a thread 128 registers (three blocks at 80 registers:
+// 112 us an adjoint stage at 128^3 against 92)
 __host__ __device__ constexpr int stage_blocks(int n, int p) {
     return 512 / ((n / p * stage_rb(n, p) + 31) / 32 * 32);
 }
@@ -502,11 +502,11 @@ __global__ void __launch_bounds__(STAGE_THREADS) k_stage(const __grid_constant__
 // current line is transformed, and the state fields of a line's products are
 // prefetched into L1 when the line begins, so that neither load stands in the
 // chain of a line's barriers.  Bound by shared memory (the LSU is 60% busy) and
-// by the barriers between a line's short steps; DRAM moves 186 MB in the
-// adjoint stage at 128^3.  Adjoint and tangent stage there: 131 us each with
+// by the barriers between a line's short steps; DRAM moves 229 MB in the
+// adjoint stage at 128^3, 241 MB in the tangent stage.  Adjoint and tangent stage there: 131 us each with
 // one line per thread as in FP64, 107 and 102 packed with run-time radices, 92
-// and 90 compiled; 5 % more with four row pairs a block, 20 % with three
-// blocks an SM (80 registers).  The last radix is small (3 to 6: the points a
+// and 90 compiled; 106 and 102 with four row pairs a block, 112 and 99 with
+// three blocks an SM (80 registers).  The last radix is small (3 to 6: the points a
 // thread holds), which leaves registers for several blocks per SM.
 __device__ __forceinline__ void put2(float* p, P2 x) { *(float2*)p = make_float2(lo(x), hi(x)); }
 __device__ __forceinline__ P2 get2(const float* p) {
@@ -1030,10 +1030,10 @@ inline bool stage_go(K kernel, const A& a, int grid, int threads, size_t smem, c
 }
 
 // Line lengths whose FP32 kernels are compiled with the length and its stage
-// radices (length, first, middle, last radix): every 5-smooth length that a
-// volume is likely to have.  Fewest stages, then the smallest largest radix,
-// then the larger last one (fewer threads a row).  Other lengths and odd
-// row counts take the kernels with run-time radices.
+// radices (length, first, middle, last radix): every 5-smooth length from 16 to
+// 320, and 384.  Fewest stages, then the smallest largest radix, then the larger
+// last one (fewer threads a row).  Other lengths and odd row counts take the
+// kernels with run-time radices.  The build compiles one unit per entry.
 #define LDDMM_STAGE_LENGTHS(X) \
     X(16, 4, 1, 4) X(18, 3, 1, 6) X(20, 4, 1, 5) X(24, 4, 1, 6) X(25, 5, 1, 5) X(27, 9, 1, 3) X(30, 5, 1, 6) \
     X(32, 8, 1, 4) X(36, 6, 1, 6) X(40, 8, 1, 5) X(45, 9, 1, 5) X(48, 8, 1, 6) X(50, 10, 1, 5) X(54, 9, 1, 6) \
