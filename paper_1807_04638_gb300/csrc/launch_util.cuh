@@ -59,8 +59,9 @@ inline int persistent_grid(int items, int per_sm = 3) {
 // ended (programmatic dependent launch): the kernel's prologue overlaps the
 // other's last blocks.  Every kernel launched this way calls after_previous()
 // before its first access to memory that another kernel of the stream writes
-// or reads, and dependents_may_launch() when it is about to write its last
-// results: at that point the launch latency and the prologue are hidden and
+// or reads, reads what the kernel in front of it wrote by plain loads (not
+// __ldg: that memory is not read-only while this kernel runs), and calls
+// dependents_may_launch() when it is about to write its last results: at that point the launch latency and the prologue are hidden and
 // the dependents take no room from its own blocks.  Hessian-vector product at
 // 64^3: 1.52 ms without, 1.42 ms so, 1.64 ms with the call at every kernel's
 // start; at 128^3 7.11, 6.97 and 6.91 ms.  k_spec_step alone calls it first: it

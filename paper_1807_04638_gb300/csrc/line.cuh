@@ -70,6 +70,13 @@ __global__ void __launch_bounds__(line_threads(N), 512 / line_threads(N)) k_line
     const bool on = l0 < lines;
     const int b0p = bd.b0p, n1 = AXIS == 1 ? N : bd.n1;
     C2* const buf = bufs + c;
+    // What the kernel in front wrote is read by plain loads from here on: it may
+    // have been written while this kernel ran, which a read-only load (__ldg)
+    // rules out and may be moved in front of the wait for.
+    auto one = [](const cpx<float>* p) {
+        const float2 v = *(const float2*)p;
+        return mk(v.x, v.y);
+    };
     after_previous();
     __syncthreads();
 
@@ -91,7 +98,7 @@ __global__ void __launch_bounds__(line_threads(N), 512 / line_threads(N)) k_line
 #pragma unroll
                     for (int r = 0; r < AA; ++r) {
                         const int c1 = LineBand<N>::template at<M>(j, r);
-                        if (c1 >= 0) v[r] = pair(__ldg((const float4*)(job.in + o0 + (unsigned)(c1 * b0p))));
+                        if (c1 >= 0) v[r] = pair(*(const float4*)(job.in + o0 + (unsigned)(c1 * b0p)));
                     }
                 } else {
                     const P2 k0v = p2(a.dk[0][ka], a.dk[0][kb]);
@@ -110,12 +117,12 @@ __global__ void __launch_bounds__(line_threads(N), 512 / line_threads(N)) k_line
                         const P2 k1v = p2(k1s, k1s);
                         C2 s;
                         if (job.kind == 1) {
-                            const C2 x0 = pair(__ldg((const float4*)(job.in + o)));
-                            const C2 x1 = pair(__ldg((const float4*)(job.in + a.cs + o)));
-                            const C2 x2 = pair(__ldg((const float4*)(job.in + 2 * a.cs + o)));
+                            const C2 x0 = pair(*(const float4*)(job.in + o));
+                            const C2 x1 = pair(*(const float4*)(job.in + a.cs + o));
+                            const C2 x2 = pair(*(const float4*)(job.in + 2 * a.cs + o));
                             s = mk(fma2(k2v, x2.x, fma2(k1v, x1.x, k0v * x0.x)), fma2(k2v, x2.y, fma2(k1v, x1.y, k0v * x0.y)));
                         } else {
-                            const C2 xa = pair(__ldg((const float4*)(pa + o))), xb = pair(__ldg((const float4*)(pb + o)));
+                            const C2 xa = pair(*(const float4*)(pa + o)), xb = pair(*(const float4*)(pb + o));
                             const P2 ua = q == 0 ? k1v : (q == 1 ? k2v : k0v), ub = q == 0 ? k2v : (q == 1 ? k0v : k1v);
                             s = mk(fma2(ua, xa.x, -(ub * xb.x)), fma2(ua, xa.y, -(ub * xb.y)));
                         }
@@ -141,7 +148,7 @@ __global__ void __launch_bounds__(line_threads(N), 512 / line_threads(N)) k_line
                 for (int r = 0; r < AA; ++r) {
                     const int kc = LineBand<N>::template at<M>(j, r);
                     if (kc >= 0) {
-                        const cpx<float> x = ldg(p0 + kc), y = ldg(p1 + kc);
+                        const cpx<float> x = one(p0 + kc), y = one(p1 + kc);
                         v[r] = mk(p2(x.x, y.x), p2(x.y, y.y));
                     }
                 }
@@ -149,20 +156,20 @@ __global__ void __launch_bounds__(line_threads(N), 512 / line_threads(N)) k_line
                 const cpx<float>* const p = job.in + (size_t)k2 * N * n1 + l0;
                 if (n1 % 2 == 0) {
 #pragma unroll
-                    for (int r = 0; r < AA; ++r) v[r] = pair(__ldg((const float4*)(p + (unsigned)((j + r * M) * n1))));
+                    for (int r = 0; r < AA; ++r) v[r] = pair(*(const float4*)(p + (unsigned)((j + r * M) * n1)));
                 } else {
                     const int d = l0 + 1 < lines ? 1 : 0;
 #pragma unroll
                     for (int r = 0; r < AA; ++r) {
                         const cpx<float>* s = p + (unsigned)((j + r * M) * n1);
-                        const cpx<float> x = ldg(s), y = ldg(s + d);
+                        const cpx<float> x = one(s), y = one(s + d);
                         v[r] = mk(p2(x.x, y.x), p2(x.y, y.y));
                     }
                 }
             } else {
                 const cpx<float>* const p = a.mid + blockIdx.z * a.mids + (unsigned)(k2 * N) * (unsigned)b0p + l0;
 #pragma unroll
-                for (int r = 0; r < AA; ++r) v[r] = pair(__ldg((const float4*)(p + (unsigned)((j + r * M) * b0p))));
+                for (int r = 0; r < AA; ++r) v[r] = pair(*(const float4*)(p + (unsigned)((j + r * M) * b0p)));
             }
         }
         dft<AA, DIR>(v);

@@ -741,6 +741,8 @@ __global__ void __launch_bounds__(NN ? (NN / P * stage_rb(NN, P) + 31) / 32 * 32
     };
 
     float* const st0 = a.state ? a.state + (size_t)m * rows + row : nullptr;
+    // read-only loads: no kernel that may still run when this one starts writes
+    // the state (a shooting's last stage is two launches and their waits earlier)
     auto S = [&](int f, int r) {
         const float* p = st0 + f * a.npts + (unsigned)(r * W) * (unsigned)rows;
         if constexpr (EVEN) return get2(p);
